@@ -96,6 +96,80 @@ def test_large_batch_and_many_rounds():
     _compare(got, ref)
 
 
+def _f32_params():
+    # the parameters as the library receives them
+    return RL.RLParams(**{n: float(np.float32(getattr(RL.RLParams(), n)))
+                          for n in ("alpha", "beta", "eta_fail", "eps", "clip_eps", "beta_h", "beta_kl")})
+
+
+def _sized_batch(rng, K, sizes=(1, 0, 3, 8, 16, 17), rounds=(0, 1, 5, 33, 70)):
+    """Groups of the given rollout counts (several warps per rollout, one, more rollouts than
+    warps), rollouts of the given round counts."""
+    correct, off = [], [0]
+    for n in sizes:
+        for _ in range(n):
+            correct.append(int(rng.random() < 0.5))
+            off.append(off[-1] + int(rng.choice(rounds)))
+    R = off[-1]
+    match = (rng.random((R, K)) < 0.6).astype(np.uint8)
+    accept = np.where(match == 1, 1, rng.random((R, K)) < 0.7).astype(np.uint8)
+    ell = (-rng.exponential(1.5, (R, K))).astype(np.float32)
+    return (np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32), np.array(correct, np.uint8),
+            np.array(off, np.int32), K, match, accept, ell)
+
+
+@pytest.mark.parametrize("policy", ["far", "near", "same", "saturated", "outside"])
+@pytest.mark.parametrize("K", [1, 31, 32, 33, 64])
+def test_sums_keep_their_precision(K, policy):
+    """The objective's sums against 64 bits at the lane and warp boundaries.  Results are 32-bit
+    roundings (6e-8); the pairs' logarithms are good to about 1e-14 absolute, the KL of two close
+    policies to 1e-9 relative, the oracle's own to about 1e-7 (p / q rounded), so 1e-6 holds for
+    every output."""
+    rng = np.random.default_rng(K)
+    batch = _sized_batch(rng, K)
+    R = batch[4].shape[0]
+    ratio = np.exp(0.3 * rng.standard_normal((R, K))).astype(np.float32)
+    p_new = rng.uniform(0.01, 0.99, (R, K)).astype(np.float32)
+    p_ref = rng.uniform(0.01, 0.99, (R, K)).astype(np.float32)
+    if policy == "near":
+        p_ref = (p_new * (1 + 1e-3 * rng.standard_normal((R, K)))).astype(np.float32)
+    elif policy == "same":
+        p_ref = p_new.copy()
+    elif policy == "saturated":
+        p_new[rng.random((R, K)) < 0.2] = 1.0
+        p_new[rng.random((R, K)) < 0.2] = 0.0
+        p_new[rng.random((R, K)) < 0.1] = 1e-9
+        p_ref[rng.random((R, K)) < 0.1] = 1e-12
+    elif policy == "outside":                # beyond the pairs' range: the 64-bit path
+        p_new[rng.random((R, K)) < 0.3] = 1e-35
+        ratio[rng.random((R, K)) < 0.2] = 1e12
+        batch[6][rng.random((R, K)) < 0.2] = -1e-20
+        batch[6][rng.random((R, K)) < 0.02] = -1e32
+    got = _run(batch, (ratio, p_new, p_ref))
+    ref = RL.rl_advantages(*batch, _f32_params(), ratio=ratio, p_new=p_new, p_ref=p_ref)
+    assert np.array_equal(got["eff"], ref["eff"])
+    for k in ("g", "rho", "J", "Jbar", "adv", "adv_dec"):
+        scale = np.nanmax(np.abs(ref[k])) if ref[k].size else 0.0
+        np.testing.assert_allclose(got[k], ref[k], rtol=1e-6, atol=1e-9 * scale, err_msg=k)
+    np.testing.assert_allclose(got["loss"], np.array(ref["loss_terms"]), rtol=1e-6, atol=0 if policy != "same" else 1e-30)
+    again = _run(batch, (ratio, p_new, p_ref))
+    assert all(np.array_equal(got[k], again[k], equal_nan=k == "rho") for k in got)
+    assert C.get_device_error() == 0
+
+
+def test_infinities_and_nan_pass_through():
+    rng = np.random.default_rng(3)
+    batch = _sized_batch(rng, 25)
+    ell = batch[6]
+    ell[rng.random(ell.shape) < 0.01] = -np.inf
+    ell[rng.random(ell.shape) < 0.005] = np.nan
+    got = _run(batch)
+    with np.errstate(all="ignore"):
+        ref = RL.rl_advantages(*batch, _f32_params())
+    for k in ("g", "rho", "J", "Jbar", "adv", "adv_dec"):
+        np.testing.assert_allclose(got[k], ref[k], rtol=1e-5, atol=1e-7, err_msg=k)
+
+
 def test_bad_offsets_set_the_error_bit_and_skip_the_group():
     rng = np.random.default_rng(5)
     go, co, ro, K, ma, ac, el = _batch(rng, 4, 5, "mixed")
