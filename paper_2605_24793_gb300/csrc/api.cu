@@ -322,7 +322,7 @@ COSPEC_API int cospec_lmhead_argmax_features(int M, int d, int V, const uint16_t
   if (!err) return cuda_lookup_failed();
   return cuda_status(launch_lmhead(M, d, V, reinterpret_cast<const __nv_bfloat16*>(hidden),
                                  reinterpret_cast<const __nv_bfloat16*>(w), draft_for_row, argmax,
-                                 stats, ws, pl, err, static_cast<cudaStream_t>(stream)));
+                                 stats, ws, LM_WS_ENTRIES, pl, err, static_cast<cudaStream_t>(stream)));
 }
 
 COSPEC_API int cospec_lmhead_sample_features(int M, int d, int V, const uint16_t* hidden,
@@ -346,7 +346,7 @@ COSPEC_API int cospec_lmhead_sample_features(int M, int d, int V, const uint16_t
   if (!err) return cuda_lookup_failed();
   return cuda_status(launch_lmhead(M, d, V, reinterpret_cast<const __nv_bfloat16*>(hidden),
                                  reinterpret_cast<const __nv_bfloat16*>(w), draft_for_row, sample,
-                                 stats, ws, pl, err, static_cast<cudaStream_t>(stream),
+                                 stats, ws, LM_WS_ENTRIES, pl, err, static_cast<cudaStream_t>(stream),
                                  reinterpret_cast<const unsigned long long*>(seed),
                                  1.0f / temperature));
 }
@@ -371,7 +371,7 @@ COSPEC_API int cospec_lmhead_logits_features(int M, int d, int V, const uint16_t
   if (!err) return cuda_lookup_failed();
   return cuda_status(launch_lmhead(M, d, V, reinterpret_cast<const __nv_bfloat16*>(hidden),
                                    reinterpret_cast<const __nv_bfloat16*>(w), draft_for_row,
-                                   argmax, stats, ws, pl, err, static_cast<cudaStream_t>(stream),
+                                   argmax, stats, ws, LM_WS_ENTRIES, pl, err, static_cast<cudaStream_t>(stream),
                                    nullptr, 1.0f / temperature, logits));
 }
 

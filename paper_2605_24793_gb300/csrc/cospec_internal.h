@@ -102,18 +102,21 @@ cudaError_t launch_verify_attn_tcq(const AttnArgs& a, const AttnPlan& plan, int*
 
 // ---------------------------------------------------------------- LM head
 struct LmheadPlan {
-  int n_mma;       // MMA N (padded rows per pass), multiple of 16, <= 256
-  int passes;      // ceil(M / 256)
-  int num_tiles;   // ceil(V / 128)
-  int grid;        // persistent CTAs
+  int n_mma;       // MMA N (padded rows per slice), multiple of 32, <= 256
+  int slices;      // ceil(M / n_mma)
+  int passes;      // row slices sharing a launch, at most 4
+  int launches;    // ceil(slices / passes)
+  int num_tiles;   // ceil(V / 256)
+  int pairs;       // CTA pairs, one CTA per SM
   int stages;
   size_t smem_bytes;
   size_t ws_bytes;
 };
+constexpr size_t LM_WS_ENTRIES = (size_t)1024 * 256;   // CTAs x rows a caller's workspace holds
 LmheadPlan plan_lmhead(int M, int d, int V, int num_sms);
 cudaError_t launch_lmhead(int M, int d, int V, const __nv_bfloat16* hidden,
                           const __nv_bfloat16* w, const int32_t* draft_for_row, int32_t* argmax,
-                          float* stats, void* ws, const LmheadPlan& plan, int* err,
+                          float* stats, void* ws, size_t ws_entries, const LmheadPlan& plan, int* err,
                           cudaStream_t stream, const unsigned long long* seed = nullptr,
                           float inv_temp = 1.f, float* logits = nullptr);
 

@@ -110,10 +110,10 @@ class VerifyRound:
 
     def _count_launches(self) -> int:
         """Kernels one round launches (attention: 1 per layer; LM head: a main
-        and a merge kernel per 256-row pass; arbitration: 1 when K > 0;
-        accept/commit: commit + scan)."""
+        and a merge kernel per launch of up to four 256-row slices;
+        arbitration: 1 when K > 0; accept/commit: commit + scan)."""
         cfg = self.cfg
-        passes = (cfg.m_rows + 255) // 256
+        passes = (cfg.m_rows + 1023) // 1024
         decide = 2 if self.sps else (1 if cfg.k > 0 else 0)
         return cfg.layers + 2 * passes + decide + 2
 

@@ -311,6 +311,81 @@ def test_lmhead_matches_oracle(case):
     print(f"lm-head {case}: tie rows {(~clear).sum()}")
 
 
+@pytest.mark.parametrize("M,d,V", [
+    (2, 64, 1),            # one id: no second logit
+    (31, 64, 100),         # the second CTA of the pair has no vocabulary row
+    (33, 128, 129),        # a second 32-column chunk; one id for the second CTA
+    (65, 192, 257),        # three chunks; a second vocabulary tile of one id
+    (257, 64, 300),        # two row slices sharing one launch
+    (1030, 64, 513),       # five slices: two launches of three and two
+])
+def test_lmhead_tile_and_slice_edges(M, d, V):
+    """Statistics, ids, logits and samples at the edges of the 256-id tiles, the 32-row chunks and the
+    row slices.  The logits are 32-bit sums of exact products (error below d ulps of the largest term
+    sum, far under the usual tolerance), so ids are compared outside near ties."""
+    rng = np.random.default_rng(M + d + V)
+    hidden, w = bf16(rng.standard_normal((M, d))), bf16(rng.standard_normal((V, d)) * 0.2)
+    dfr = rng.integers(-1, V, M).astype(np.int32)
+    dfr_t = torch.from_numpy(dfr).cuda()
+    ids = torch.empty(M, dtype=torch.int32, device="cuda")
+    st = torch.empty((M, 5), dtype=torch.float32, device="cuda")
+    ws = C.new_lmhead_workspace(M, d, V)
+    x = O.lmhead_logits(host(hidden), host(w))
+    with np.errstate(all="ignore"):
+        ref_am, ref_st = O.lmhead_stats(host(hidden), host(w), dfr)
+    if V == 1:
+        ref_st[:, 1] = -np.inf
+        ref_st[:, 3] = 0.0
+    clear = ref_st[:, 0] - ref_st[:, 1] >= 1e-3
+    logits = torch.empty((M, V), dtype=torch.float32, device="cuda")
+    for mode in ("greedy", "logits"):
+        if mode == "greedy":
+            C.lmhead_argmax_features(hidden, w, dfr_t, ids, st, ws)
+        else:
+            C.lmhead_logits_features(hidden, w, dfr_t, 1.0, ids, st, logits, ws)
+            assert_close(logits.cpu().numpy(), x, "logits")
+        got = st.cpu().numpy()
+        assert np.array_equal(np.isinf(got[:, 1]), np.isinf(ref_st[:, 1]))
+        fin = ref_st.copy()
+        fin[:, 1] = np.where(np.isinf(fin[:, 1]), 0, fin[:, 1])
+        got[:, 1] = np.where(np.isinf(got[:, 1]), 0, got[:, 1])
+        assert_close(got, fin, f"{mode} stats")
+        assert np.array_equal(ids.cpu().numpy()[clear], ref_am[clear])
+    seed = 0x5DEECE66D1234567
+    C.lmhead_sample_features(hidden, w, dfr_t, 1.0, torch.tensor([seed], dtype=torch.int64, device="cuda"), ids, st, ws)
+    keys = O.gumbel_keys(x, seed, 1.0)
+    sure = np.ones(M, bool) if V == 1 else np.diff(np.sort(keys, axis=1)[:, -2:], axis=1)[:, 0] >= 1e-3
+    assert np.array_equal(ids.cpu().numpy()[sure], np.argmax(keys, axis=1)[sure])
+    assert C.get_device_error() == 0
+
+
+def test_lmhead_extreme_logits():
+    """Equal logits and a logit near the largest float keep well-defined statistics; NaN is passed on."""
+    M, d, V = 40, 64, 700
+    hidden = np.zeros((M, d), np.float32)
+    w = np.zeros((V, d), np.float32)
+    w[:, 0] = 1.0
+    w[7, 1] = 1.0                       # the only id that sees column 1
+    hidden[1, 0] = 3.0                  # all logits 3
+    hidden[2, 1] = 1e38                 # one huge logit: the others underflow
+    hidden[3, 1] = np.inf               # inf * 0: NaN logits beside an infinite one
+    hidden[4, 2] = 1e38
+    w[650, 2] = 1e38                    # overflows to one infinite logit in row 4
+    hidden_t, w_t = bf16(hidden), bf16(w)
+    ids = torch.empty(M, dtype=torch.int32, device="cuda")
+    st = torch.empty((M, 5), dtype=torch.float32, device="cuda")
+    C.lmhead_argmax_features(hidden_t, w_t, torch.full((M,), 7, dtype=torch.int32, device="cuda"), ids, st,
+                             C.new_lmhead_workspace(M, d, V))
+    ids, st = ids.cpu().numpy(), st.cpu().numpy()
+    assert ids[0] == 0 and ids[1] == 0 and ids[2] == 7
+    np.testing.assert_allclose(st[0, :4], [0, 0, np.log(V), np.log(V)], rtol=1e-6)
+    np.testing.assert_allclose(st[1], [3, 3, 3 + np.log(V), np.log(V), 3], rtol=1e-6)
+    np.testing.assert_allclose(st[2], [st[2, 4], 0, st[2, 4], 0, st[2, 4]], rtol=1e-6)
+    assert np.isnan(st[3, 2])           # NaN logits reach the log-sum-exp
+    assert ids[4] == 650 and st[4, 0] == np.inf and st[4, 2] == np.inf
+    assert C.get_device_error() == 0
+
+
 def test_lmhead_exact_ties_pick_lowest_id():
     rng = np.random.default_rng(11)
     M, d, V = 8, 256, 700
