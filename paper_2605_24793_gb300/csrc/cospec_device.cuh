@@ -348,7 +348,10 @@ CS_DEV void named_bar_sync(int id, int nthreads) {
 
 // Batches up to this size are taken longest context first (the ranking below
 // reads every context length once per candidate pass, O(B^2 / 32) per CTA);
-// larger batches, enough units for many waves, are taken in index order.
+// larger batches, enough units for many waves, are taken in index order (the
+// tcgen05 kernel: in reverse when the last context is longer than the first, as
+// with the chunks of a prefill in their own order, whose long ones should start
+// early).
 constexpr int RANK_MAX_B = 64;
 
 // The sequence whose context is the `z`-th longest (ties to the lower index):
@@ -384,6 +387,10 @@ CS_DEV int sequence_by_rank(const int32_t* ctx_len, int B, int z, volatile int* 
   return b;
 }
 
+// The sequence of the launch's z-th slot in a batch above RANK_MAX_B.
+CS_DEV int sequence_in_order(const int32_t* ctx_len, int B, int z) {
+  return ctx_len[B - 1] > ctx_len[0] ? B - 1 - z : z;
+}
 
 // Philox4x32-10: ten rounds of two 32x32 -> 64-bit products by the
 // multipliers 0xD2511F53 / 0xCD9E8D57, the key advanced by the Weyl

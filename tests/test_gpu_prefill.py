@@ -32,6 +32,9 @@ def _bf16(rng, shape):
     (1, 1, 33, 32, 8, 128, 17),      # one full chunk and one row, K = 7 region
     (1, 3, 96, 16, 8, 128, 53),      # three full chunks, K = 25 region (53 rows)
     (1, 1, 1000, 8, 2, 128, 17),     # 32 chunks, the last of 8 rows
+    (2, 3, 704, 4, 2, 64, 9),        # whole chunks, read where they lie: 66 chunk sequences, two layers
+    (1, 2, 256, 2, 2, 64, 9),        # one query head per KV head, whole blocks of 64
+    (1, 2, 200, 2, 2, 64, 9),        # the same, ragged and an odd number of chunks
 ])
 def test_prefill_then_region_matches_dense_hybrid_attention(method, L, B, T, Hq, Hkv, D, region):
     rng = np.random.default_rng(T * 7 + region)
