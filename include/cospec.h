@@ -119,7 +119,7 @@ COSPEC_API int cospec_num_sms(void);
  *    distributed shared memory.  Two kernels implement the call: one on
  *    mma.sync tensor-core tiles, and one on tcgen05 (TMEM accumulators, the
  *    query rows as the MMA M dimension, up to 128 rows of a KV head per
- *    CTA), used when a KV head has more than 32 query rows (and at most 64
+ *    CTA, or 256 sharing each K/V tile), used when a KV head has more than 32 query rows (and at most 64
  *    query heads share the KV head).  Batches of up to 64 sequences are
  *    processed longest context first; larger ones in index order (tcgen05:
  *    in reverse when the last context is longer than the first; a caller can

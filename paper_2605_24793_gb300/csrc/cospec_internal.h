@@ -80,8 +80,10 @@ struct AttnArgs {
 struct AttnPlan {
   int kind;               // 0: mma.sync kernel, 1: tcgen05 kernel (query rows as MMA M)
   int mt, wk, nrp;        // mma.sync: row tiles, key groups, padded rows
-  int nt, jb, jbq, rg;    // tcgen05: row capacity (128), block rows per row group,
-                          // block rows of the query box, row groups
+  int nt, jb, jbq, rg;    // tcgen05: row capacity of a row tile (128), block rows per row
+                          // tile, block rows of the query box, row groups
+  int two;                // tcgen05: a row group is two row tiles sharing the cache stream
+  int jg;                 // tcgen05: block rows per row group
   int cluster;            // CTAs per (sequence, KV head, row group): the KV split
   long long units;        // (sequence, KV head, row group) units, one cluster each
   int one_wave;           // small batch: take the largest split whose clusters are
@@ -95,6 +97,8 @@ AttnPlan plan_verify_attn(int B, int R, int Hq, int Hkv, int D, int max_ctx, int
 int attn_max_active_clusters(int D, int mt, int wk, int S, int Hkv, int B, int kbr);
 cudaError_t launch_verify_attn(const AttnArgs& a, const AttnPlan& plan, int* err,
                                cudaStream_t stream);
+cudaError_t launch_verify_attn_tcq2(const AttnArgs& a, const AttnPlan& plan, int* err,
+                                    cudaStream_t stream);
 bool tcq_attn_supported(int D, int G);
 int attn_tcq_max_active_clusters(int D, int S, int Hkv, int B, int RG);
 cudaError_t launch_verify_attn_tcq(const AttnArgs& a, const AttnPlan& plan, int* err,

@@ -13,25 +13,28 @@
 //   warps 0-2  TMA producers: 128-key K/V tiles (one 2-D box per page and
 //              128-byte half: [half][128 keys][128 B], 128B-swizzled) into a
 //              3-stage ring, the block's own K/V as a final tile;
-//   warp 3     MMA issuer (one thread), which first loads the query rows of
+//   warp 3     MMA issuer (one elected thread), which first loads the query rows of
 //              the group:
-//                S  = Q K^T   (M = 128 query rows, N = 128 keys, K = D) into
-//                             one of three TMEM score buffers,
-//                O += P V     (M = 128 query rows, N = D, K = keys) with P
-//                             read from TMEM (written over its score
-//                             buffer; three buffers, so S may run two
-//                             tiles ahead of P.V) and V read MN-major from
-//                             the V tile;
+//                S    = Q K^T  (M = 128 query rows, N = 128 keys, K = D) into
+//                              one of two TMEM score buffers,
+//                O_h += P_h V  (M = 128 query rows, N = D, K = 64 keys) for each
+//                              key half h with P_h read from TMEM (written over
+//                              its scores) and V read MN-major from the V tile;
 //   warps 4-11 softmax, two groups of four warps (one per TMEM lane quarter)
-//              sharing every tile, group g its key columns 64 g .. 64 g + 63:
-//              a thread owns one query row and half of its scores; the two
-//              threads of a row swap their half maxima through shared memory,
-//              turn their scores into bf16 P in place and rescale their half
-//              of the row of O when the row's reference maximum moves.
-// Softmax with a lazy reference maximum per row: scores are taken relative
-// to m_ref, set exactly by the first tile; a later tile moves m_ref (and
-// rescales O and l) only when one of its scores exceeds m_ref by more than
+//              sharing every tile, group h its key columns 64 h .. 64 h + 63: a
+//              thread owns one query row and half of its scores, with a reference
+//              maximum, a sum and an output accumulator O_h of its own, so nothing
+//              passes between the groups until the two halves of a row are put
+//              together at the end.
+// Softmax with a lazy reference maximum per row and half: scores are taken
+// relative to m_ref, set exactly by the first tile; a later tile moves m_ref (and
+// rescales O_h and l) only when one of its scores exceeds it by more than
 // 2^8 in the exp2 domain, so P stays below 256 and rescales are rare.
+// What bounds it: a tile's 32 boxes of 2 KB enter an SM about 58 cycles apart however many
+// warps issue them (1900 cycles per 128-key tile, 10.7 TB/s over the chip), above the HBM
+// share.  Measured (GB300, us per layer) against the two halves swapping their maxima
+// through shared memory (2250 cycles per tile): Qwen3-32B batch 32, K = 7: 176 -> 172;
+// Qwen3-8B batch 16, K = 25: 63.9 -> 63.6.
 #include <cuda.h>
 #include <math.h>
 
@@ -80,14 +83,13 @@ struct TcqLayout {
   static constexpr int QH = QM * QROWB;             // one half of the query rows
   static constexpr int QOFF = RING;
   static constexpr int MISC = QOFF + H * QH;
-  // barriers: full_k[NS], full_v[NS], empty_k[NS], empty_v[NS], q_full, s_full[NSB],
-  // p_full[NSB], pv_done, mma_done, recv_bar
-  static constexpr int NSB = 3;                     // TMEM score buffers
-  static constexpr int NBAR = 4 * NS + 2 * NSB + 4;
+  // barriers: full_k[NS], full_v[NS], empty_k[NS], empty_v[NS], q_full, s_full[2],
+  // p_full[2 buffers][2 halves], pv_done[2 halves], mma_done, recv_bar
+  static constexpr int NSB = 2;                     // TMEM score buffers
+  static constexpr int NBAR = 4 * NS + 11;
   static constexpr int HOLDER = MISC + NBAR * 8;    // TMEM base address
-  static constexpr int FLAGS = HOLDER + 16;         // abort, tiles issued [2], sequence slot, row-pair votes [8]
-  static constexpr int XCH = FLAGS + 64;            // float [2][QM]: the groups' row maxima / sums
-  static constexpr int TOTAL = XCH + 2 * QM * 4;
+  static constexpr int FLAGS = HOLDER + 16;         // abort, tiles issued [2], sequence slot
+  static constexpr int TOTAL = FLAGS + 16;
   // partial rows after the last tile, in the idle ring: PART [QM], RECV [QM + 15]
   static constexpr int PD = D + 4;                  // O[D], m, l, pad: conflict-free row stores
   static constexpr int ROWP = PD * 4;
@@ -95,62 +97,11 @@ struct TcqLayout {
   static constexpr int RECV = QM * ROWP;
   static_assert(RECV + (QM + 15) * ROWP <= RING, "partials must fit in the ring");
   static_assert(ROWP % 16 == 0, "bulk copies move whole 16-byte chunks");
-  // TMEM columns: score buffers at 0, 128 and 256, O at 384
+  // TMEM columns: score buffers at 0 and 128, O_0 and O_1 from 256
   static constexpr uint32_t TCOLS = 512u;
   static constexpr uint32_t OCOL = NSB * QKT;
-  static_assert(OCOL + D <= TCOLS, "the O accumulator after the score buffers");
+  static_assert(OCOL + 2 * D <= TCOLS, "two O accumulators after the score buffers");
 };
-
-// 32 lanes x 32 bit, 16 consecutive columns per thread (no wait).
-CS_DEV void tq_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-      "%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-CS_DEV void tq_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-CS_DEV void tq_st16(uint32_t taddr, const uint32_t* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15,%16};" ::"r"(taddr),
-      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-      "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]),
-      "r"(v[15])
-      : "memory");
-}
-CS_DEV void tq_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-// D[tmem] (+)= A[tmem] * B[smem desc], bf16 inputs, fp32 accumulate.  A is
-// M x 16 with row m in TMEM lane m and two bf16 per 32-bit column.
-CS_DEV void umma_bf16_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                             uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Descriptor of an MN-major operand in the 128B-swizzle layout: 64-element
-// rows of 128 bytes along MN, consecutive rows = consecutive K; `lbo` bytes
-// between the 64-element groups along MN, 1024 bytes between 8-row groups
-// along K.
-CS_DEV uint64_t tq_desc_mn_sw128(uint32_t saddr, uint32_t lbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
 
 template <int D>
 __global__ void __launch_bounds__(Q_THREADS, 1)
@@ -176,15 +127,14 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   uint64_t* empty_v = empty_k + NS;
   uint64_t* q_full = empty_v + NS;
   uint64_t* s_full = q_full + 1;      // [NSB]
-  uint64_t* p_full = s_full + LY::NSB;  // [NSB]
-  uint64_t* pv_done = p_full + LY::NSB;
-  uint64_t* mma_done = pv_done + 1;
+  uint64_t* p_full = s_full + LY::NSB;  // [NSB][2 halves]
+  uint64_t* pv_done = p_full + 2 * LY::NSB;   // [2 halves]
+  uint64_t* mma_done = pv_done + 2;
   uint64_t* recv_bar = mma_done + 1;  // partials received from the cluster
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + LY::HOLDER);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + LY::FLAGS);
   volatile int* n_issued = abort_flag + 1;   // [2]: tiles whose K / V loads were issued (abort tail)
   volatile int* seq_slot = abort_flag + 3;
-  volatile int* xvote = abort_flag + 4;      // [2 groups][4 quarters]: this tile's waits succeeded
   uint8_t* qs = smem + LY::QOFF;
 
   const int S = (int)cluster_nctarank();
@@ -207,9 +157,11 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     mbar_init(q_full, 1);
     for (int i = 0; i < LY::NSB; ++i) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&p_full[i], (uint32_t)(2 * nsw));   // both softmax groups' warps with rows
+      mbar_init(&p_full[2 * i], (uint32_t)nsw);     // a softmax group's warps with rows
+      mbar_init(&p_full[2 * i + 1], (uint32_t)nsw);
     }
-    mbar_init(pv_done, 1);
+    mbar_init(&pv_done[0], 1);
+    mbar_init(&pv_done[1], 1);
     mbar_init(mma_done, 1);
     mbar_init(recv_bar, 1);
     abort_flag[0] = 0;
@@ -362,72 +314,89 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     if (pw != 1 && lane == 0) n_issued[tensor] = issued;
   } else if (warp == Q_MMA_WARP) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && T > 0) {
+    // (the whole warp walks along; one elected thread acts)
+    if (T > 0) {
+      const uint32_t on = elect_one();
       const uint32_t idesc_pv = idesc_bf16_f32(QM, D) | (1u << 16);   // B (V) MN-major
-      const uint32_t q0 = smem_u32(qs);
-      {
-        // The query rows come from the previous kernel: this thread loads
-        // them as soon as that kernel is done, while the producer warps are
-        // still issuing the first cache tiles (a warp's bulk copies run one
-        // after another; behind three tiles' boxes the rows landed ~2 us
-        // later at batch 1).
-        if (p.kv_stable) griddep_wait();
+      // The query rows come from the previous kernel: this warp loads them as
+      // soon as that kernel is done, while the producer warps are still issuing
+      // the first cache tiles (a warp's bulk copies run one after another; behind
+      // three tiles' boxes the rows landed ~2 us later at batch 1).
+      if (p.kv_stable) griddep_wait();
+      if (on) {
         const uint64_t qpol = p.RG > 1 ? l2_policy_evict_normal() : l2_policy_evict_first();
         mbar_arrive_expect_tx(q_full, (uint32_t)(H * qrows * QROWB));
         for (int h = 0; h < H; ++h)
           tma_load_4d(smem_u32(qs + h * LY::QH), &map_q, q_full, 0, kvh * p.G, b * p.R + j0, h, qpol);
       }
-      bool ok = mbar_wait(q_full, 0, Q_WAIT_NS);
+      __syncwarp();
+      const uint32_t sbase = smem_u32(smem);
+      const uint64_t q_desc = smem_desc_sw128(sbase + LY::QOFF);
+      const uint64_t k_desc = smem_desc_sw128(sbase);
+      bool ok = __all_sync(0xffffffffu, mbar_wait(q_full, 0, Q_WAIT_NS));
+      // (descriptor addresses count 16-byte units)
       auto issue_s = [&](int t) {
         const int st = t % NS;
-        const uint32_t kb = smem_u32(smem + st * LY::STAGE);
-        const bool blk = do_blk && t == n;
-        const int nk = blk ? KBR : QKT;
-        const uint32_t khalf = (uint32_t)(nk * QROWB);
+        const int nk = (do_blk && t == n) ? KBR : QKT;
+        const uint64_t kd = k_desc + (uint64_t)(st * (LY::STAGE >> 4));
+        const uint64_t khalf = (uint64_t)(nk * (QROWB >> 4));
         const uint32_t idesc_qk = idesc_bf16_f32(QM, nk);
+        const uint32_t dst = tmem_base + (uint32_t)((t & 1) * QKT);
 #pragma unroll
         for (int h = 0; h < H; ++h)
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)
-            umma_bf16(tmem_base + (uint32_t)((t % LY::NSB) * QKT), smem_desc_sw128(q0 + h * LY::QH + ks * 32),
-                      smem_desc_sw128(kb + h * khalf + ks * 32), idesc_qk, (h | ks) != 0 ? 1u : 0u);
-        umma_commit(&empty_k[st]);         // K of this stage is free once S is done
-        umma_commit(&s_full[t % LY::NSB]);
+            umma_bf16_on(on, dst, q_desc + (uint64_t)(h * (LY::QH >> 4) + ks * 2),
+                         kd + h * khalf + (uint64_t)(ks * 2), idesc_qk, (h | ks) != 0 ? 1u : 0u);
+        umma_commit_on(on, &empty_k[st]);         // K of this stage is free once S is done
+        umma_commit_on(on, &s_full[t & 1]);
       };
-      auto issue_pv = [&](int u) {
-        const int st = u % NS;
-        const uint32_t vb = smem_u32(smem + st * LY::STAGE + LY::KVB);
-        const bool blk = do_blk && u == n;
-        const int nk = blk ? KBR : QKT;
-        const uint32_t vhalf = (uint32_t)(nk * QROWB);
-        // P of tile u: 16 keys = 8 TMEM columns per step
-        for (int ks = 0; ks < nk / 16; ++ks)
-          umma_bf16_tmem_a(tmem_base + LY::OCOL,
-                           tmem_base + (uint32_t)((u % LY::NSB) * QKT + ks * 8),
-                           tq_desc_mn_sw128(vb + ks * 2048, vhalf), idesc_pv,
-                           (u > 0 || ks > 0) ? 1u : 0u);
-        umma_commit(&empty_v[st]);
-        umma_commit(pv_done);
-      };
-      // Issue whichever product is ready, so that a P.V product (which frees
-      // a ring stage for the producer) never waits behind the next tile's
-      // load.  S of tile ts goes to buffer ts % 3, last read (as P) by the
-      // P.V product of tile ts - 3: tcgen05 MMAs of one thread run in issue
-      // order, so S may be issued once that product is.  At most two tiles'
-      // S run ahead of the oldest pending P.V, which also keeps every
-      // barrier within one phase of the parity tested here.
-      int ts = 0, tp = 0, idle = 0;
-      uint64_t t_last = global_timer_ns();
-      while (ok && tp < T) {
-        bool did = false;
-        if (tp < ts && mbar_test(&p_full[tp % LY::NSB], (uint32_t)(tp / LY::NSB) & 1u) &&
-            mbar_test(&full_v[tp % NS], (uint32_t)(tp / NS) & 1u)) {
-          tc_fence_after();
-          issue_pv(tp);
-          ++tp;
-          did = true;
+      // O_h += P_h V over keys 64 h .. of tile u (the block tile is all in half 0)
+      auto issue_pv = [&](int u, int h) {
+        const uint32_t vb = sbase + (uint32_t)((u % NS) * LY::STAGE + LY::KVB + h * (64 * QROWB));
+        const uint32_t src = tmem_base + (uint32_t)((u & 1) * QKT + h * 64);
+        const uint32_t dst = tmem_base + LY::OCOL + (uint32_t)(h * D);
+        // 16 keys = 8 TMEM columns and 16 rows of V (2 KB) per MMA
+        if (do_blk && u == n) {
+          const uint64_t vd = tq_desc_mn_sw128(vb, (uint32_t)(KBR * QROWB));
+          for (int ks = 0; ks < KBR / 16; ++ks)
+            umma_bf16_tmem_a_on(on, dst, src + (uint32_t)(ks * 8), vd + (uint64_t)(ks * 128), idesc_pv,
+                                (u > 0 || ks > 0) ? 1u : 0u);
+        } else {
+          const uint64_t vd = tq_desc_mn_sw128(vb, (uint32_t)(QKT * QROWB));
+          const uint32_t acc0 = u > 0 ? 1u : 0u;
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks)
+            umma_bf16_tmem_a_on(on, dst, src + (uint32_t)(ks * 8), vd + (uint64_t)(ks * 128), idesc_pv,
+                                ks > 0 ? 1u : acc0);
         }
-        if (ts < T && ts <= tp + 2 && mbar_test(&full_k[ts % NS], (uint32_t)(ts / NS) & 1u)) {
+        umma_commit_on(on, &pv_done[h]);
+      };
+      // Issue whichever product is ready.  S of tile ts goes to buffer ts & 1, last
+      // read (as P) by the P.V products of tile ts - 2: tcgen05 MMAs of one thread
+      // run in issue order, so S may be issued once those are.  That also keeps
+      // every barrier within one phase of the parity tested here.
+      int ts = 0, tp0 = 0, tp1 = 0, idle = 0;
+      uint64_t t_last = global_timer_ns();
+      while (ok && (tp0 < T || tp1 < n)) {
+        bool did = false;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          int& tp = h ? tp1 : tp0;
+          const int other = h ? tp0 : tp1;
+          if (tp < (h ? n : T) && tp < ts &&
+              __all_sync(0xffffffffu, mbar_test(&p_full[2 * (tp & 1) + h], (uint32_t)(tp >> 1) & 1u) &&
+                                          mbar_test(&full_v[tp % NS], (uint32_t)(tp / NS) & 1u))) {
+            tc_fence_after();
+            issue_pv(tp, h);
+            // V of this stage is free once both halves' products are done
+            if (other > tp || tp == n) umma_commit_on(on, &empty_v[tp % NS]);
+            ++tp;
+            did = true;
+          }
+        }
+        if (ts < T && ts <= tp0 + 1 && (ts <= tp1 + 1) &&
+            __all_sync(0xffffffffu, mbar_test(&full_k[ts % NS], (uint32_t)(ts / NS) & 1u))) {
           tc_fence_after();
           issue_s(ts);
           ++ts;
@@ -439,34 +408,29 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
         } else if ((++idle & 255) == 0) {
           const uint64_t now = global_timer_ns();
           if (idle == 256) t_last = now;
-          else if (*abort_flag || now - t_last > Q_WAIT_NS) ok = false;
+          else if (__any_sync(0xffffffffu, *abort_flag || now - t_last > Q_WAIT_NS)) ok = false;
         }
       }
-      if (!ok) {
+      if (!ok && on) {
         set_err(p.err, ERR_TIMEOUT);
         *abort_flag = 1;
       }
-      // every MMA issued by this thread completes before TMEM is released
-      umma_commit(mma_done);
+      // every MMA issued by this warp's thread completes before TMEM is released
+      umma_commit_on(on, mma_done);
       mbar_wait(mma_done, 0, Q_WAIT_NS);
     }
   } else {
     // ------------------------------------------------------------ softmax
     // Two groups of four warps (one warp per TMEM lane quarter each) share
-    // every tile: group g takes its key columns 64 g .. 64 g + 63.  A thread
-    // owns one query row; the two threads of a row (same lane, warps q and
-    // q + 4) swap their half-tile maxima through shared memory, so both move
-    // the row's reference maximum together and their P, written over their
-    // own columns of the score buffer, share one O accumulator.
+    // every tile: group h takes its key columns 64 h .. 64 h + 63.  A thread
+    // owns one query row and its half of the keys.
     const int sw = warp - Q_SOFT0;
     const int grp = sw >> 2;             // key-column half of every tile
     const int q = sw & 3;                // TMEM lane quarter of this warp
     const int r = q * 32 + lane;         // this thread's query row
-    const int gtid = q * 32 + lane;      // thread index within the group
     const int kc0 = grp * (QKT / 2);     // first key column of this half
-    float* xch = reinterpret_cast<float*>(smem + LY::XCH);   // [2][QM]
     if (p.kv_stable) {
-      // warm L2 with the group's query rows before the producer's TMA
+      // warm L2 with the group's query rows before the MMA warp's loads
       for (int e = sw * 32 + lane; e < NR * (D * 2 / 128); e += 256) {
         const int rr = e / (D * 2 / 128), part_ = e % (D * 2 / 128);
         const int j = j0 + rr / p.G, g = rr % p.G;
@@ -479,63 +443,46 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     const int blim = p.block_full ? p.R - 1 : min(jr, p.R - 1);
     const float sc = p.scale_log2;
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
-    const uint32_t ocol = LY::OCOL + (uint32_t)(grp * (D / 2));   // this group's half of O
-    constexpr int HK = QKT / 2;          // key columns of a half
+    const uint32_t ocol = LY::OCOL + (uint32_t)(grp * D);   // this half's O
+    const int T_mine = grp ? n : T;      // the block tile's keys are all in half 0
     if (q < nsw) {
-      for (int t = 0; t < T; ++t) {
-        const int sb_i = t % LY::NSB;
-        const int st = t % NS;
-        uint8_t* sb = smem + st * LY::STAGE;
+      for (int t = 0; t < T_mine; ++t) {
         const bool blk = do_blk && t == n;
-        const int nk = blk ? KBR : QKT;          // score columns of this tile
-        // The two warps of a row pair decide an abort together (from both
-        // votes, read after the first exchange barrier), so neither is left
-        // waiting at a barrier the other no longer reaches.
-        const bool okw =
-            __all_sync(0xffffffffu, mbar_wait(&s_full[sb_i], (uint32_t)(t / LY::NSB) & 1u, Q_WAIT_NS)) &&
-            !*abort_flag;
-        if (lane == 0) xvote[grp * 4 + q] = okw ? 1 : 0;
-        tc_fence_after();
-        const uint32_t srow = lane_base + (uint32_t)(sb_i * QKT);
-        // keys 0..lim of this tile are visible to this row (raw scores; the
-        // scale is positive, so it is applied with the exponent).  Padding
-        // rows (r >= NR) give rows of P and O that nothing reads, so they
-        // decide neither the masking nor a rescale.
-        const int lim = blk ? blim : min(QKT, C - (t_begin + t) * QKT) - 1;
-        float x[HK];
-#pragma unroll
-        for (int c = 0; c < HK / 16; ++c) {
-          if (okw && kc0 + c * 16 < nk) {
-            tq_ld16(srow + kc0 + c * 16, &x[c * 16]);
-          } else {
-#pragma unroll
-            for (int k = 0; k < 16; ++k) x[c * 16 + k] = -INFINITY;
-          }
-        }
-        tq_wait_ld();
-        if (__any_sync(0xffffffffu, rvalid && lim < kc0 + HK - 1)) {
-#pragma unroll
-          for (int k = 0; k < HK; ++k) x[k] = (kc0 + k <= lim) ? x[k] : -INFINITY;
-        }
-        float m4[4] = {x[0], x[1], x[2], x[3]};
-#pragma unroll
-        for (int k = 4; k < HK; ++k) m4[k & 3] = fmaxf(m4[k & 3], x[k]);
-        const float mh = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-        // the row's maximum over both halves (both threads have read their
-        // scores by the first barrier, so P may then overwrite them; the
-        // second barrier lets the buffer be rewritten at the next tile)
-        xch[grp * QM + r] = mh;
-        named_bar_sync(1 + q, 64);
-        const float mx = fmaxf(mh, xch[(grp ^ 1) * QM + r]) * sc;
-        const bool ok2 = xvote[q] != 0 && xvote[4 + q] != 0;
-        named_bar_sync(1 + q, 64);
-        if (!ok2) {
+        const int nk = blk ? KBR : QKT / 2;      // score columns of this half
+        if (!__all_sync(0xffffffffu, mbar_wait(&s_full[t & 1], (uint32_t)(t >> 1) & 1u, Q_WAIT_NS)) || *abort_flag) {
           if (lane == 0) {
             set_err(p.err, ERR_TIMEOUT);
             *abort_flag = 1;
           }
           break;
         }
+        tc_fence_after();
+        const uint32_t srow = lane_base + (uint32_t)((t & 1) * QKT + kc0);
+        // keys 0..lim of this half are visible to this row (raw scores; the
+        // scale is positive, so it is applied with the exponent).  Padding
+        // rows (r >= NR) give rows of P and O that nothing reads, so they
+        // decide neither the masking nor a rescale.  A block tile has 16 to 64
+        // score columns; the rest of the half holds an earlier tile's.
+        const int left = C - (t_begin + t) * QKT - kc0;      // context keys from here on
+        const int lim = blk ? blim : min(QKT / 2, left) - 1;
+        float x0[32], x1[32];
+        tq_ld32(srow, x0);
+        tq_ld32(srow + 32, x1);
+        tq_wait_ld32(x0);
+        tq_wait_ld32(x1);
+        if (__any_sync(0xffffffffu, rvalid && lim < QKT / 2 - 1) || blk) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k) {
+            x0[k] = k <= lim ? x0[k] : -INFINITY;
+            x1[k] = 32 + k <= lim ? x1[k] : -INFINITY;
+          }
+        }
+        float m4[4] = {x0[0], x0[1], x0[2], x0[3]};
+#pragma unroll
+        for (int k = 4; k < 32; ++k) m4[k & 3] = fmaxf(m4[k & 3], x0[k]);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) m4[k & 3] = fmaxf(m4[k & 3], x1[k]);
+        const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * sc;
         // move the reference only when a score exceeds it by 2^8 (the first
         // tile always sets it: m_ref starts at -inf)
         const bool up = rvalid && mx > mref + Q_LAZY;
@@ -546,14 +493,13 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
           l *= alpha;
         }
         if (__any_sync(0xffffffffu, up && t > 0)) {
-          // O holds tiles 0..t-1: wait for the last of them, then scale this
-          // group's half of the row
+          // O_h holds tiles 0..t-1: wait for the last of them, then scale the row
           const bool okp =
-              __all_sync(0xffffffffu, mbar_wait(pv_done, (uint32_t)(t - 1) & 1u, Q_WAIT_NS));
+              __all_sync(0xffffffffu, mbar_wait(&pv_done[grp], (uint32_t)(t - 1) & 1u, Q_WAIT_NS));
           tc_fence_after();
           if (okp) {
 #pragma unroll 1
-            for (int c = 0; c < D / 32; ++c) {
+            for (int c = 0; c < D / 16; ++c) {
               float o[16];
               tq_ld16(lane_base + ocol + c * 16, o);
               tq_wait_ld();
@@ -566,32 +512,34 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
             set_err(p.err, ERR_TIMEOUT);
           }
         }
-        // P = 2^(score * scale - m_ref) in bf16, two keys per TMEM column, in
-        // this half's columns of the score buffer (masked keys give exactly 0)
+        // P = 2^(score * scale - m_ref) in bf16, two keys per TMEM column, over
+        // this half's scores (masked keys give exactly 0)
         const float nb = (mref == -INFINITY) ? 0.f : -mref;
         float l4[4] = {0.f, 0.f, 0.f, 0.f};
-        uint32_t pk[HK / 2];
+        auto exp_store = [&](float (&x)[32], int k0) {
+          uint32_t pk[16];
 #pragma unroll
-        for (int k = 0; k < HK / 2; ++k) {
-          const float p0 = exp2_approx(fmaf(x[2 * k], sc, nb));
-          const float p1 = exp2_approx(fmaf(x[2 * k + 1], sc, nb));
-          l4[k & 3] += p0 + p1;
-          pk[k] = pack_bf16(p0, p1);
-        }
+          for (int k = 0; k < 16; ++k) {
+            const float p0 = exp2_approx(fmaf(x[2 * k], sc, nb));
+            const float p1 = exp2_approx(fmaf(x[2 * k + 1], sc, nb));
+            l4[k & 3] += p0 + p1;
+            pk[k] = pack_bf16(p0, p1);
+          }
+          tq_st16(srow + k0 / 2, pk);
+        };
+        exp_store(x0, 0);
+        exp_store(x1, 32);
         l += (l4[0] + l4[1]) + (l4[2] + l4[3]);
-#pragma unroll
-        for (int c = 0; c < HK / 32; ++c)
-          if (kc0 + c * 32 < nk) tq_st16(srow + kc0 / 2 + c * 16, &pk[c * 16]);
         // V rows of keys outside the context (or past the block) may hold
-        // stale bytes: group 0 zeroes them so that their zero weights
+        // stale bytes: the half's group zeroes them so that their zero weights
         // contribute 0 (V lands separately from K: wait for it first).
-        if (grp == 0) {
-          const int vr = blk ? p.R : min(QKT, C - (t_begin + t) * QKT);
-          if (vr < nk &&
-              __all_sync(0xffffffffu, mbar_wait(&full_v[st], (uint32_t)(t / NS) & 1u, Q_WAIT_NS))) {
-            uint8_t* vb = sb + LY::KVB;
-            const int vhalf = nk * QROWB;
-            for (int e = gtid; e < (nk - vr) * H * 8; e += nsw * 32) {
+        const int vr = blk ? p.R : min(QKT / 2, max(0, left));
+        if (vr < nk) {
+          const int st = t % NS;
+          if (__all_sync(0xffffffffu, mbar_wait(&full_v[st], (uint32_t)(t / NS) & 1u, Q_WAIT_NS))) {
+            uint8_t* vb = smem + st * LY::STAGE + LY::KVB + kc0 * QROWB;
+            const int vhalf = (blk ? KBR : QKT) * QROWB;
+            for (int e = r; e < (nk - vr) * H * 8; e += nsw * 32) {
               const int row = vr + e / (H * 8), rem = e % (H * 8);
               *reinterpret_cast<uint4*>(vb + (rem / 8) * vhalf + row * QROWB + (rem % 8) * 16) =
                   make_uint4(0u, 0u, 0u, 0u);
@@ -602,28 +550,25 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
         tq_wait_st();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&p_full[sb_i]);
+        if (lane == 0) mbar_arrive(&p_full[2 * (t & 1) + grp]);
       }
-      if (T > 0 && !*abort_flag) {
+      if (T_mine > 0 && !*abort_flag) {
         const bool okp =
-            __all_sync(0xffffffffu, mbar_wait(pv_done, (uint32_t)(T - 1) & 1u, Q_WAIT_NS));
+            __all_sync(0xffffffffu, mbar_wait(&pv_done[grp], (uint32_t)(T_mine - 1) & 1u, Q_WAIT_NS));
         if (!okp && lane == 0) {
           set_err(p.err, ERR_TIMEOUT);
           *abort_flag = 1;
         }
       }
-      tc_fence_after();
-    }
-    // the row's sum over both halves (the exchange buffer is free: every
-    // tile's second barrier has passed)
-    if (q < nsw) {
-      xch[grp * QM + r] = l;
-      named_bar_sync(1 + q, 64);
-      l += xch[(grp ^ 1) * QM + r];
+      tc_fence_before();
     }
   }
   __syncthreads();
   tc_fence_after();
+  // Every MMA is done: the query rows' place takes the (m_ref, l) of the row halves.
+  float2* ml = reinterpret_cast<float2*>(qs);                // [2 halves][QM]
+  if (warp >= Q_SOFT0) ml[tid - Q_SOFT0 * 32] = make_float2(mref, l);
+  __syncthreads();
 
   // ---------------------------------------------------------------- output
   // The ring is idle from here on.  Unsplit, every softmax thread writes its
@@ -638,19 +583,27 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   }
   float* part = reinterpret_cast<float*>(smem + LY::PART);
   if (warp >= Q_SOFT0 && ((warp - Q_SOFT0) & 3) < nsw) {
-    // each group writes its half of the row's columns (both hold m_ref and l)
+    // The two halves of a row are put together: common maximum, weighted sums.
+    // Each group writes half of the row's columns.
     const int sw = warp - Q_SOFT0, grp = sw >> 2, q = sw & 3, r = q * 32 + lane;
     const bool rvalid = r < NR;
     const int c0 = grp * (D / 32);       // first 16-column chunk of this group's half
     const uint32_t orow = tmem_base + ((uint32_t)(q * 32) << 16) + LY::OCOL;
+    const float2 h0 = ml[r], h1 = ml[QM + r];
+    mref = fmaxf(h0.x, h1.x);
+    const float w0_ = (h0.x == -INFINITY) ? 0.f : exp2_approx(h0.x - mref);
+    const float w1_ = (h1.x == -INFINITY) ? 0.f : exp2_approx(h1.x - mref);
+    l = h0.y * w0_ + h1.y * w1_;
+    const bool have1 = have && n > 0;    // half 1 holds cache tiles only
     auto load_o = [&](int c, float (&o)[16]) {
+      float o1[16];
       if (have) {
         tq_ld16(orow + c * 16, o);
+        if (have1) tq_ld16(orow + D + c * 16, o1);
         tq_wait_ld();
-      } else {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) o[i] = 0.f;
       }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) o[i] = have ? (have1 ? o[i] * w0_ + o1[i] * w1_ : o[i] * w0_) : 0.f;
     };
     if (S == 1) {
       const int j = j0 + (rvalid ? r / p.G : 0), g = rvalid ? r % p.G : 0;
@@ -773,9 +726,11 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   }
 }
 
+// At least 118 KB, so that two CTAs (each wants all of TMEM) never share an SM.
 template <int D>
 size_t tcq_smem_bytes() {
-  return (size_t)TcqLayout<D>::TOTAL + 1024;
+  const size_t need = (size_t)TcqLayout<D>::TOTAL + 1024;
+  return need > 118 * 1024 ? need : 118 * 1024;
 }
 
 // Limits already set on each instantiation of the kernel.

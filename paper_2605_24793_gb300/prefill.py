@@ -81,16 +81,16 @@ class BlockPrefill:
         self.tokens = torch.zeros(B2 * R, dtype=torch.int32, device=dev)
         self.s = torch.empty(B2, dtype=torch.int32, device=dev)
         self.emitted = torch.empty((B2, R), dtype=torch.int32, device=dev)
-        # The attention may take several chunks as one block (up to 64 rows).
-        # With one query head per KV head a chunk alone would be small enough
-        # for the mma.sync kernel, which takes the chunks first to last.
+        # The attention takes several chunks as one block where they divide the
+        # context (up to 64 rows; up to 256 query rows share a KV head's cache
+        # stream).
         self.rows = chunk
-        if q_heads == kv_heads and (self.nck * chunk) % (64 // chunk * chunk) == 0:
-            self.rows = 64 // chunk * chunk
-        blocks = self.nck * chunk // self.rows
-        self.block_table = torch.from_numpy(np.repeat(table, blocks, axis=0)).to(dev)
-        self.block_start = torch.from_numpy(
-            np.tile(np.arange(blocks, dtype=np.int32) * self.rows, batch)).to(dev)
+        most = 64 // chunk * chunk
+        if (self.nck * chunk) % most == 0 and q_heads // kv_heads * most <= 256:
+            self.rows = most
+        step = self.rows // chunk
+        self.block_table = self.table2[::step].contiguous()
+        self.block_start = self.start[::step].contiguous()
         # chunk-padded projections [L, B, nck * chunk, H, D], made by the first load()
         self.qp = self.kp = self.vp = self.outp = None
 

@@ -175,6 +175,60 @@ def test_verify_attention_tcgen05_split_matches_oracle(case):
     assert_close(host(out), ref, "attention (tcgen05, split)")
 
 
+# Contexts around the edges of pages, 64-key softmax steps and 128-key tiles.
+EDGE_CTX = [0, 1, 15, 16, 63, 64, 65, 100, 127, 128, 129, 191, 192, 193, 255, 300]
+
+
+@pytest.mark.parametrize("full", [False, True], ids=["causal", "full"])
+@pytest.mark.parametrize("R,Hq,Hkv,D", [
+    (33, 32, 8, 128),     # 132 rows: the second row tile has four
+    (53, 32, 8, 128),     # 212 rows
+    (64, 32, 8, 64),      # 256 rows, head_dim 64
+    (64, 24, 8, 128),     # G = 3: row tiles of 42 block rows (126 query rows)
+    (40, 64, 8, 128),     # G = 8: a group of two row tiles and one of a single tile
+    (20, 32, 8, 128),     # 80 rows: the one-tile kernel, unsplit
+    (32, 16, 8, 64),      # 64 rows, head_dim 64
+])
+def test_verify_attention_tile_edges(R, Hq, Hkv, D, full):
+    """One and two row tiles per CTA at every key remainder (more than 128 rows on 128 or more
+    (sequence, head) units of a few tiles take two).  bf16 outputs of probabilities rounded to bf16:
+    the usual tolerance."""
+    B = len(EDGE_CTX)
+    rng = np.random.default_rng(R * 100 + Hq + D)
+    t = _paged_case(rng, B, R, Hq, Hkv, D, EDGE_CTX, True)
+    assert C.verify_attn_plan(t["q"], t["k_pages"], t["page_table"], max(EDGE_CTX)) == (C.ATTN_TCGEN05, 1)
+    out = torch.empty_like(t["q"])
+    C.verify_attn(t["q"], t["k_blk"], t["v_blk"], t["k_pages"], t["v_pages"], t["page_table"],
+                  t["ctx_len"], out, max(EDGE_CTX), block_full=full)
+    ref = O.verify_attention(host(t["q"]), host(t["k_blk"]), host(t["v_blk"]), host(t["k_pages"]),
+                             host(t["v_pages"]), t["table_np"], t["ctx_np"], 16,
+                             **({"block_mask": "full"} if full else {}))
+    assert_close(host(out), ref, "attention (tile edges)")
+    assert C.get_device_error() == 0
+
+
+@pytest.mark.parametrize("R", [20, 53])
+def test_verify_attention_moving_maximum(R):
+    """Scores that grow along the context move the reference maximum (and rescale the outputs) tile
+    after tile, in one half of the keys and not the other."""
+    B, Hq, Hkv, D = 16, 32, 8, 128
+    ctx = [40 * (i + 1) for i in range(B)]
+    rng = np.random.default_rng(R)
+    t = _paged_case(rng, B, R, Hq, Hkv, D, ctx, False)
+    table = t["table_np"]
+    for b in range(B):
+        for pos in range(ctx[b]):
+            scale = 0.2 + 0.02 * pos if (pos // 64) % 2 == 0 else 0.1
+            t["k_pages"][int(table[b, pos // 16]), :, pos % 16] *= scale
+    t["q"] *= 2
+    out = torch.empty_like(t["q"])
+    C.verify_attn(t["q"], t["k_blk"], t["v_blk"], t["k_pages"], t["v_pages"], t["page_table"],
+                  t["ctx_len"], out, max(ctx))
+    ref = O.verify_attention(host(t["q"]), host(t["k_blk"]), host(t["v_blk"]), host(t["k_pages"]),
+                             host(t["v_pages"]), t["table_np"], t["ctx_np"], 16)
+    assert_close(host(out), ref, "attention (moving maximum)")
+
+
 # The arbitrator's draft/target region (Sec. 3.3): 2K+3 block rows that see
 # the whole block; K = 7 gives 17 rows, K = 25 (the paper's default) 53.
 ATTN_FULL_CASES = [
