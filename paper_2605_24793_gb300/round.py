@@ -111,11 +111,11 @@ class VerifyRound:
     def _count_launches(self) -> int:
         """Kernels one round launches (attention: 1 per layer; LM head: a main
         and a merge kernel per launch of up to four 256-row slices;
-        arbitration: 1 when K > 0; accept/commit: commit + scan)."""
+        arbitration: 1 when K > 0; accept/commit: 1)."""
         cfg = self.cfg
         passes = (cfg.m_rows + 1023) // 1024
         decide = 2 if self.sps else (1 if cfg.k > 0 else 0)
-        return cfg.layers + 2 * passes + decide + 2
+        return cfg.layers + 2 * passes + decide + 1
 
     def restore_context(self) -> None:
         """Reset ctx_len to the round's starting context (device copy)."""
