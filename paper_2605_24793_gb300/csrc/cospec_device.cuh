@@ -322,6 +322,14 @@ CS_DEV void tq_st16(uint32_t taddr, const uint32_t* v) {
       "r"(v[15])
       : "memory");
 }
+// Two 32-bit columns per thread: store, and load with its wait.
+CS_DEV void tq_st2(uint32_t taddr, float a, float b) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "f"(a), "f"(b) : "memory");
+}
+CS_DEV void tq_ld2(uint32_t taddr, float& a, float& b) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(a), "+f"(b)::"memory");
+}
 CS_DEV void tq_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // D[tmem] (+)= A[tmem] * B[smem desc], bf16 inputs, fp32 accumulate.  A is

@@ -30,11 +30,15 @@
 // relative to m_ref, set exactly by the first tile; a later tile moves m_ref (and
 // rescales O_h and l) only when one of its scores exceeds it by more than
 // 2^8 in the exp2 domain, so P stays below 256 and rescales are rare.
+// With SWAP (clusters of eight or more CTAs: a few tiles each) the two threads of a row swap
+// their half maxima through shared memory every tile instead and share one reference,
+// sum and accumulator O, with a third score buffer in the room that is left; nothing is
+// left to put together at the end.
 // What bounds it: a tile's 32 boxes of 2 KB enter an SM about 58 cycles apart however many
 // warps issue them (1900 cycles per 128-key tile, 10.7 TB/s over the chip), above the HBM
-// share.  Measured (GB300, us per layer) against the two halves swapping their maxima
-// through shared memory (2250 cycles per tile): Qwen3-32B batch 32, K = 7: 176 -> 172;
-// Qwen3-8B batch 16, K = 25: 63.9 -> 63.6.
+// share.  Measured (GB300, us per layer back to back), swapping -> independent halves (2250 ->
+// 1900 cycles per tile): Qwen3-32B batch 32, K = 7: 173.6 -> 171.6; Qwen3-8B batch 4,
+// K = 25: 19.2 -> 18.9; 212-row regions, batch 8, 4096 keys 42.4 -> 39.9.
 #include <cuda.h>
 #include <math.h>
 
@@ -73,7 +77,7 @@ struct TcqParams {
   int* err;
 };
 
-template <int D>
+template <int D, bool SWAP>
 struct TcqLayout {
   static constexpr int H = D / 64;                  // 128-byte halves of a key row
   static constexpr int KVB = H * QKT * QROWB;       // K (or V) of a tile: [half][128 keys][128 B]
@@ -83,13 +87,14 @@ struct TcqLayout {
   static constexpr int QH = QM * QROWB;             // one half of the query rows
   static constexpr int QOFF = RING;
   static constexpr int MISC = QOFF + H * QH;
-  // barriers: full_k[NS], full_v[NS], empty_k[NS], empty_v[NS], q_full, s_full[2],
-  // p_full[2 buffers][2 halves], pv_done[2 halves], mma_done, recv_bar
-  static constexpr int NSB = 2;                     // TMEM score buffers
-  static constexpr int NBAR = 4 * NS + 11;
+  // barriers: full_k[NS], full_v[NS], empty_k[NS], empty_v[NS], q_full, s_full[NSB],
+  // p_full[NSB][2 halves], pv_done[2 halves], mma_done, recv_bar
+  static constexpr int NSB = SWAP ? 3 : 2;          // TMEM score buffers
+  static constexpr int NBAR = 4 * NS + 3 * NSB + 5;
   static constexpr int HOLDER = MISC + NBAR * 8;    // TMEM base address
-  static constexpr int FLAGS = HOLDER + 16;         // abort, tiles issued [2], sequence slot
-  static constexpr int TOTAL = FLAGS + 16;
+  static constexpr int FLAGS = HOLDER + 16;         // abort, tiles issued [2], sequence slot, votes [8]
+  static constexpr int XCH = FLAGS + 48;            // SWAP: float [2][QM], the groups' row maxima / sums
+  static constexpr int TOTAL = XCH + (SWAP ? 2 * QM * 4 : 0);
   // partial rows after the last tile, in the idle ring: PART [QM], RECV [QM + 15]
   static constexpr int PD = D + 4;                  // O[D], m, l, pad: conflict-free row stores
   static constexpr int ROWP = PD * 4;
@@ -97,20 +102,20 @@ struct TcqLayout {
   static constexpr int RECV = QM * ROWP;
   static_assert(RECV + (QM + 15) * ROWP <= RING, "partials must fit in the ring");
   static_assert(ROWP % 16 == 0, "bulk copies move whole 16-byte chunks");
-  // TMEM columns: score buffers at 0 and 128, O_0 and O_1 from 256
+  // TMEM columns: score buffers from 0, then O (SWAP) or O_0 and O_1
   static constexpr uint32_t TCOLS = 512u;
   static constexpr uint32_t OCOL = NSB * QKT;
-  static_assert(OCOL + 2 * D <= TCOLS, "two O accumulators after the score buffers");
+  static_assert(OCOL + (SWAP ? 1 : 2) * D <= TCOLS, "the O accumulators after the score buffers");
 };
 
-template <int D>
+template <int D, bool SWAP>
 __global__ void __launch_bounds__(Q_THREADS, 1)
     verify_attn_tcq_kernel(const __grid_constant__ CUtensorMap map_kp,
                            const __grid_constant__ CUtensorMap map_vp,
                            const __grid_constant__ CUtensorMap map_kb,
                            const __grid_constant__ CUtensorMap map_vb,
                            const __grid_constant__ CUtensorMap map_q, const TcqParams p) {
-  using LY = TcqLayout<D>;
+  using LY = TcqLayout<D, SWAP>;
   constexpr int H = LY::H;
   constexpr int NS = LY::NS;
   constexpr int PD = LY::PD;
@@ -135,6 +140,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + LY::FLAGS);
   volatile int* n_issued = abort_flag + 1;   // [2]: tiles whose K / V loads were issued (abort tail)
   volatile int* seq_slot = abort_flag + 3;
+  volatile int* xvote = abort_flag + 4;      // SWAP: [2 groups][4 quarters], this tile's waits succeeded
   uint8_t* qs = smem + LY::QOFF;
 
   const int S = (int)cluster_nctarank();
@@ -157,7 +163,8 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     mbar_init(q_full, 1);
     for (int i = 0; i < LY::NSB; ++i) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&p_full[2 * i], (uint32_t)nsw);     // a softmax group's warps with rows
+      // a softmax group's warps with rows (SWAP: both groups', on the first of the two)
+      mbar_init(&p_full[2 * i], (uint32_t)(SWAP ? 2 * nsw : nsw));
       mbar_init(&p_full[2 * i + 1], (uint32_t)nsw);
     }
     mbar_init(&pv_done[0], 1);
@@ -314,110 +321,204 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     if (pw != 1 && lane == 0) n_issued[tensor] = issued;
   } else if (warp == Q_MMA_WARP) {
     // ------------------------------------------------------------ MMA issuer
-    // (the whole warp walks along; one elected thread acts)
-    if (T > 0) {
-      const uint32_t on = elect_one();
-      const uint32_t idesc_pv = idesc_bf16_f32(QM, D) | (1u << 16);   // B (V) MN-major
-      // The query rows come from the previous kernel: this warp loads them as
-      // soon as that kernel is done, while the producer warps are still issuing
-      // the first cache tiles (a warp's bulk copies run one after another; behind
-      // three tiles' boxes the rows landed ~2 us later at batch 1).
-      if (p.kv_stable) griddep_wait();
-      if (on) {
-        const uint64_t qpol = p.RG > 1 ? l2_policy_evict_normal() : l2_policy_evict_first();
-        mbar_arrive_expect_tx(q_full, (uint32_t)(H * qrows * QROWB));
-        for (int h = 0; h < H; ++h)
-          tma_load_4d(smem_u32(qs + h * LY::QH), &map_q, q_full, 0, kvh * p.G, b * p.R + j0, h, qpol);
-      }
-      __syncwarp();
-      const uint32_t sbase = smem_u32(smem);
-      const uint64_t q_desc = smem_desc_sw128(sbase + LY::QOFF);
-      const uint64_t k_desc = smem_desc_sw128(sbase);
-      bool ok = __all_sync(0xffffffffu, mbar_wait(q_full, 0, Q_WAIT_NS));
-      // (descriptor addresses count 16-byte units)
-      auto issue_s = [&](int t) {
-        const int st = t % NS;
-        const int nk = (do_blk && t == n) ? KBR : QKT;
-        const uint64_t kd = k_desc + (uint64_t)(st * (LY::STAGE >> 4));
-        const uint64_t khalf = (uint64_t)(nk * (QROWB >> 4));
-        const uint32_t idesc_qk = idesc_bf16_f32(QM, nk);
-        const uint32_t dst = tmem_base + (uint32_t)((t & 1) * QKT);
-#pragma unroll
-        for (int h = 0; h < H; ++h)
-#pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            umma_bf16_on(on, dst, q_desc + (uint64_t)(h * (LY::QH >> 4) + ks * 2),
-                         kd + h * khalf + (uint64_t)(ks * 2), idesc_qk, (h | ks) != 0 ? 1u : 0u);
-        umma_commit_on(on, &empty_k[st]);         // K of this stage is free once S is done
-        umma_commit_on(on, &s_full[t & 1]);
-      };
-      // O_h += P_h V over keys 64 h .. of tile u (the block tile is all in half 0)
-      auto issue_pv = [&](int u, int h) {
-        const uint32_t vb = sbase + (uint32_t)((u % NS) * LY::STAGE + LY::KVB + h * (64 * QROWB));
-        const uint32_t src = tmem_base + (uint32_t)((u & 1) * QKT + h * 64);
-        const uint32_t dst = tmem_base + LY::OCOL + (uint32_t)(h * D);
-        // 16 keys = 8 TMEM columns and 16 rows of V (2 KB) per MMA
-        if (do_blk && u == n) {
-          const uint64_t vd = tq_desc_mn_sw128(vb, (uint32_t)(KBR * QROWB));
-          for (int ks = 0; ks < KBR / 16; ++ks)
-            umma_bf16_tmem_a_on(on, dst, src + (uint32_t)(ks * 8), vd + (uint64_t)(ks * 128), idesc_pv,
-                                (u > 0 || ks > 0) ? 1u : 0u);
-        } else {
-          const uint64_t vd = tq_desc_mn_sw128(vb, (uint32_t)(QKT * QROWB));
-          const uint32_t acc0 = u > 0 ? 1u : 0u;
-#pragma unroll
-          for (int ks = 0; ks < 4; ++ks)
-            umma_bf16_tmem_a_on(on, dst, src + (uint32_t)(ks * 8), vd + (uint64_t)(ks * 128), idesc_pv,
-                                ks > 0 ? 1u : acc0);
+    if constexpr (SWAP) {
+      if (lane == 0 && T > 0) {
+        const uint32_t idesc_pv = idesc_bf16_f32(QM, D) | (1u << 16);   // B (V) MN-major
+        const uint32_t q0 = smem_u32(qs);
+        {
+          // The query rows come from the previous kernel: this thread loads
+          // them as soon as that kernel is done, while the producer warps are
+          // still issuing the first cache tiles (a warp's bulk copies run one
+          // after another; behind three tiles' boxes the rows landed ~2 us
+          // later at batch 1).
+          if (p.kv_stable) griddep_wait();
+          const uint64_t qpol = p.RG > 1 ? l2_policy_evict_normal() : l2_policy_evict_first();
+          mbar_arrive_expect_tx(q_full, (uint32_t)(H * qrows * QROWB));
+          for (int h = 0; h < H; ++h)
+            tma_load_4d(smem_u32(qs + h * LY::QH), &map_q, q_full, 0, kvh * p.G, b * p.R + j0, h, qpol);
         }
-        umma_commit_on(on, &pv_done[h]);
-      };
-      // Issue whichever product is ready.  S of tile ts goes to buffer ts & 1, last
-      // read (as P) by the P.V products of tile ts - 2: tcgen05 MMAs of one thread
-      // run in issue order, so S may be issued once those are.  That also keeps
-      // every barrier within one phase of the parity tested here.
-      int ts = 0, tp0 = 0, tp1 = 0, idle = 0;
-      uint64_t t_last = global_timer_ns();
-      while (ok && (tp0 < T || tp1 < n)) {
-        bool did = false;
+        bool ok = mbar_wait(q_full, 0, Q_WAIT_NS);
+        auto issue_s = [&](int t) {
+          const int st = t % NS;
+          const uint32_t kb = smem_u32(smem + st * LY::STAGE);
+          const bool blk = do_blk && t == n;
+          const int nk = blk ? KBR : QKT;
+          const uint32_t khalf = (uint32_t)(nk * QROWB);
+          const uint32_t idesc_qk = idesc_bf16_f32(QM, nk);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          int& tp = h ? tp1 : tp0;
-          const int other = h ? tp0 : tp1;
-          if (tp < (h ? n : T) && tp < ts &&
-              __all_sync(0xffffffffu, mbar_test(&p_full[2 * (tp & 1) + h], (uint32_t)(tp >> 1) & 1u) &&
-                                          mbar_test(&full_v[tp % NS], (uint32_t)(tp / NS) & 1u))) {
+          for (int h = 0; h < H; ++h)
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+              umma_bf16(tmem_base + (uint32_t)((t % LY::NSB) * QKT), smem_desc_sw128(q0 + h * LY::QH + ks * 32),
+                        smem_desc_sw128(kb + h * khalf + ks * 32), idesc_qk, (h | ks) != 0 ? 1u : 0u);
+          umma_commit(&empty_k[st]);         // K of this stage is free once S is done
+          umma_commit(&s_full[t % LY::NSB]);
+        };
+        auto issue_pv = [&](int u) {
+          const int st = u % NS;
+          const uint32_t vb = smem_u32(smem + st * LY::STAGE + LY::KVB);
+          const bool blk = do_blk && u == n;
+          const int nk = blk ? KBR : QKT;
+          const uint32_t vhalf = (uint32_t)(nk * QROWB);
+          // P of tile u: 16 keys = 8 TMEM columns per step
+          for (int ks = 0; ks < nk / 16; ++ks)
+            umma_bf16_tmem_a(tmem_base + LY::OCOL,
+                             tmem_base + (uint32_t)((u % LY::NSB) * QKT + ks * 8),
+                             tq_desc_mn_sw128(vb + ks * 2048, vhalf), idesc_pv,
+                             (u > 0 || ks > 0) ? 1u : 0u);
+          umma_commit(&empty_v[st]);
+          umma_commit(&pv_done[0]);
+        };
+        // Issue whichever product is ready, so that a P.V product (which frees
+        // a ring stage for the producer) never waits behind the next tile's
+        // load.  S of tile ts goes to buffer ts % 3, last read (as P) by the
+        // P.V product of tile ts - 3: tcgen05 MMAs of one thread run in issue
+        // order, so S may be issued once that product is.  At most two tiles'
+        // S run ahead of the oldest pending P.V, which also keeps every
+        // barrier within one phase of the parity tested here.
+        int ts = 0, tp = 0, idle = 0;
+        uint64_t t_last = global_timer_ns();
+        while (ok && tp < T) {
+          bool did = false;
+          if (tp < ts && mbar_test(&p_full[2 * (tp % LY::NSB)], (uint32_t)(tp / LY::NSB) & 1u) &&
+              mbar_test(&full_v[tp % NS], (uint32_t)(tp / NS) & 1u)) {
             tc_fence_after();
-            issue_pv(tp, h);
-            // V of this stage is free once both halves' products are done
-            if (other > tp || tp == n) umma_commit_on(on, &empty_v[tp % NS]);
+            issue_pv(tp);
             ++tp;
             did = true;
           }
+          if (ts < T && ts <= tp + 2 && mbar_test(&full_k[ts % NS], (uint32_t)(ts / NS) & 1u)) {
+            tc_fence_after();
+            issue_s(ts);
+            ++ts;
+            did = true;
+          }
+          // the clock is read only every 256 idle polls (the limit stays bounded)
+          if (did) {
+            idle = 0;
+          } else if ((++idle & 255) == 0) {
+            const uint64_t now = global_timer_ns();
+            if (idle == 256) t_last = now;
+            else if (*abort_flag || now - t_last > Q_WAIT_NS) ok = false;
+          }
         }
-        if (ts < T && ts <= tp0 + 1 && (ts <= tp1 + 1) &&
-            __all_sync(0xffffffffu, mbar_test(&full_k[ts % NS], (uint32_t)(ts / NS) & 1u))) {
-          tc_fence_after();
-          issue_s(ts);
-          ++ts;
-          did = true;
+        if (!ok) {
+          set_err(p.err, ERR_TIMEOUT);
+          *abort_flag = 1;
         }
-        // the clock is read only every 256 idle polls (the limit stays bounded)
-        if (did) {
-          idle = 0;
-        } else if ((++idle & 255) == 0) {
-          const uint64_t now = global_timer_ns();
-          if (idle == 256) t_last = now;
-          else if (__any_sync(0xffffffffu, *abort_flag || now - t_last > Q_WAIT_NS)) ok = false;
-        }
+        // every MMA issued by this thread completes before TMEM is released
+        umma_commit(mma_done);
+        mbar_wait(mma_done, 0, Q_WAIT_NS);
       }
-      if (!ok && on) {
-        set_err(p.err, ERR_TIMEOUT);
-        *abort_flag = 1;
+    } else {
+      // (the whole warp walks along; one elected thread acts)
+      if (T > 0) {
+        const uint32_t on = elect_one();
+        const uint32_t idesc_pv = idesc_bf16_f32(QM, D) | (1u << 16);   // B (V) MN-major
+        // The query rows come from the previous kernel: this warp loads them as
+        // soon as that kernel is done, while the producer warps are still issuing
+        // the first cache tiles (a warp's bulk copies run one after another; behind
+        // three tiles' boxes the rows landed ~2 us later at batch 1).
+        if (p.kv_stable) griddep_wait();
+        if (on) {
+          const uint64_t qpol = p.RG > 1 ? l2_policy_evict_normal() : l2_policy_evict_first();
+          mbar_arrive_expect_tx(q_full, (uint32_t)(H * qrows * QROWB));
+          for (int h = 0; h < H; ++h)
+            tma_load_4d(smem_u32(qs + h * LY::QH), &map_q, q_full, 0, kvh * p.G, b * p.R + j0, h, qpol);
+        }
+        __syncwarp();
+        const uint32_t sbase = smem_u32(smem);
+        const uint64_t q_desc = smem_desc_sw128(sbase + LY::QOFF);
+        const uint64_t k_desc = smem_desc_sw128(sbase);
+        bool ok = __all_sync(0xffffffffu, mbar_wait(q_full, 0, Q_WAIT_NS));
+        // (descriptor addresses count 16-byte units)
+        auto issue_s = [&](int t) {
+          const int st = t % NS;
+          const int nk = (do_blk && t == n) ? KBR : QKT;
+          const uint64_t kd = k_desc + (uint64_t)(st * (LY::STAGE >> 4));
+          const uint64_t khalf = (uint64_t)(nk * (QROWB >> 4));
+          const uint32_t idesc_qk = idesc_bf16_f32(QM, nk);
+          const uint32_t dst = tmem_base + (uint32_t)((t & 1) * QKT);
+#pragma unroll
+          for (int h = 0; h < H; ++h)
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+              umma_bf16_on(on, dst, q_desc + (uint64_t)(h * (LY::QH >> 4) + ks * 2),
+                           kd + h * khalf + (uint64_t)(ks * 2), idesc_qk, (h | ks) != 0 ? 1u : 0u);
+          umma_commit_on(on, &empty_k[st]);         // K of this stage is free once S is done
+          umma_commit_on(on, &s_full[t & 1]);
+        };
+        // O_h += P_h V over keys 64 h .. of tile u (the block tile is all in half 0)
+        auto issue_pv = [&](int u, int h) {
+          const uint32_t vb = sbase + (uint32_t)((u % NS) * LY::STAGE + LY::KVB + h * (64 * QROWB));
+          const uint32_t src = tmem_base + (uint32_t)((u & 1) * QKT + h * 64);
+          const uint32_t dst = tmem_base + LY::OCOL + (uint32_t)(h * D);
+          // 16 keys = 8 TMEM columns and 16 rows of V (2 KB) per MMA
+          if (do_blk && u == n) {
+            const uint64_t vd = tq_desc_mn_sw128(vb, (uint32_t)(KBR * QROWB));
+            for (int ks = 0; ks < KBR / 16; ++ks)
+              umma_bf16_tmem_a_on(on, dst, src + (uint32_t)(ks * 8), vd + (uint64_t)(ks * 128), idesc_pv,
+                                  (u > 0 || ks > 0) ? 1u : 0u);
+          } else {
+            const uint64_t vd = tq_desc_mn_sw128(vb, (uint32_t)(QKT * QROWB));
+            const uint32_t acc0 = u > 0 ? 1u : 0u;
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+              umma_bf16_tmem_a_on(on, dst, src + (uint32_t)(ks * 8), vd + (uint64_t)(ks * 128), idesc_pv,
+                                  ks > 0 ? 1u : acc0);
+          }
+          umma_commit_on(on, &pv_done[h]);
+        };
+        // Issue whichever product is ready.  S of tile ts goes to buffer ts & 1, last
+        // read (as P) by the P.V products of tile ts - 2: tcgen05 MMAs of one thread
+        // run in issue order, so S may be issued once those are.  That also keeps
+        // every barrier within one phase of the parity tested here.
+        int ts = 0, tp0 = 0, tp1 = 0, idle = 0;
+        uint64_t t_last = global_timer_ns();
+        while (ok && (tp0 < T || tp1 < n)) {
+          // every barrier in question is tested at once (a test changes nothing)
+          const bool p0 = mbar_test(&p_full[2 * (tp0 & 1)], (uint32_t)(tp0 >> 1) & 1u);
+          const bool p1 = mbar_test(&p_full[2 * (tp1 & 1) + 1], (uint32_t)(tp1 >> 1) & 1u);
+          const bool v0 = mbar_test(&full_v[tp0 % NS], (uint32_t)(tp0 / NS) & 1u);
+          const bool v1 = mbar_test(&full_v[tp1 % NS], (uint32_t)(tp1 / NS) & 1u);
+          const bool ks = mbar_test(&full_k[ts % NS], (uint32_t)(ts / NS) & 1u);
+          const bool go0 = __all_sync(0xffffffffu, (tp0 < T) & (tp0 < ts) & p0 & v0);
+          const bool go1 = __all_sync(0xffffffffu, (tp1 < n) & (tp1 < ts) & p1 & v1);
+          const bool gos = __all_sync(0xffffffffu, (ts < T) & (ts <= tp0 + 1) & (ts <= tp1 + 1) & ks);
+          const bool did = go0 | go1 | gos;
+          if (did) tc_fence_after();
+          if (go0) {
+            issue_pv(tp0, 0);
+            // V of this stage is free once both halves' products are done
+            if (tp1 > tp0 || tp0 == n) umma_commit_on(on, &empty_v[tp0 % NS]);
+            ++tp0;
+          }
+          if (go1) {
+            issue_pv(tp1, 1);
+            if (tp0 > tp1) umma_commit_on(on, &empty_v[tp1 % NS]);
+            ++tp1;
+          }
+          if (gos) {
+            issue_s(ts);
+            ++ts;
+          }
+          // the clock is read only every 256 idle polls (the limit stays bounded)
+          if (did) {
+            idle = 0;
+          } else if ((++idle & 255) == 0) {
+            const uint64_t now = global_timer_ns();
+            if (idle == 256) t_last = now;
+            else if (__any_sync(0xffffffffu, *abort_flag || now - t_last > Q_WAIT_NS)) ok = false;
+          }
+        }
+        if (!ok && on) {
+          set_err(p.err, ERR_TIMEOUT);
+          *abort_flag = 1;
+        }
+        // every MMA issued by this warp's thread completes before TMEM is released
+        umma_commit_on(on, mma_done);
+        mbar_wait(mma_done, 0, Q_WAIT_NS);
       }
-      // every MMA issued by this warp's thread completes before TMEM is released
-      umma_commit_on(on, mma_done);
-      mbar_wait(mma_done, 0, Q_WAIT_NS);
     }
   } else {
     // ------------------------------------------------------------ softmax
@@ -443,200 +544,354 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     const int blim = p.block_full ? p.R - 1 : min(jr, p.R - 1);
     const float sc = p.scale_log2;
     const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
-    const uint32_t ocol = LY::OCOL + (uint32_t)(grp * D);   // this half's O
-    const int T_mine = grp ? n : T;      // the block tile's keys are all in half 0
-    if (q < nsw) {
-      for (int t = 0; t < T_mine; ++t) {
-        const bool blk = do_blk && t == n;
-        const int nk = blk ? KBR : QKT / 2;      // score columns of this half
-        if (!__all_sync(0xffffffffu, mbar_wait(&s_full[t & 1], (uint32_t)(t >> 1) & 1u, Q_WAIT_NS)) || *abort_flag) {
-          if (lane == 0) {
-            set_err(p.err, ERR_TIMEOUT);
-            *abort_flag = 1;
-          }
-          break;
-        }
-        tc_fence_after();
-        const uint32_t srow = lane_base + (uint32_t)((t & 1) * QKT + kc0);
-        // keys 0..lim of this half are visible to this row (raw scores; the
-        // scale is positive, so it is applied with the exponent).  Padding
-        // rows (r >= NR) give rows of P and O that nothing reads, so they
-        // decide neither the masking nor a rescale.  A block tile has 16 to 64
-        // score columns; the rest of the half holds an earlier tile's.
-        const int left = C - (t_begin + t) * QKT - kc0;      // context keys from here on
-        const int lim = blk ? blim : min(QKT / 2, left) - 1;
-        float x0[32], x1[32];
-        tq_ld32(srow, x0);
-        tq_ld32(srow + 32, x1);
-        tq_wait_ld32(x0);
-        tq_wait_ld32(x1);
-        if (__any_sync(0xffffffffu, rvalid && lim < QKT / 2 - 1) || blk) {
-#pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            x0[k] = k <= lim ? x0[k] : -INFINITY;
-            x1[k] = 32 + k <= lim ? x1[k] : -INFINITY;
-          }
-        }
-        float m4[4] = {x0[0], x0[1], x0[2], x0[3]};
-#pragma unroll
-        for (int k = 4; k < 32; ++k) m4[k & 3] = fmaxf(m4[k & 3], x0[k]);
-#pragma unroll
-        for (int k = 0; k < 32; ++k) m4[k & 3] = fmaxf(m4[k & 3], x1[k]);
-        const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * sc;
-        // move the reference only when a score exceeds it by 2^8 (the first
-        // tile always sets it: m_ref starts at -inf)
-        const bool up = rvalid && mx > mref + Q_LAZY;
-        float alpha = 1.f;
-        if (up) {
-          alpha = (mref == -INFINITY) ? 0.f : exp2_approx(mref - mx);
-          mref = mx;
-          l *= alpha;
-        }
-        if (__any_sync(0xffffffffu, up && t > 0)) {
-          // O_h holds tiles 0..t-1: wait for the last of them, then scale the row
-          const bool okp =
-              __all_sync(0xffffffffu, mbar_wait(&pv_done[grp], (uint32_t)(t - 1) & 1u, Q_WAIT_NS));
+    // this half's O (SWAP: its columns of the one O)
+    const uint32_t ocol = LY::OCOL + (uint32_t)(grp * (SWAP ? D / 2 : D));
+    if constexpr (SWAP) {
+      // The row's two halves share one reference maximum, sum and accumulator.
+      float* xch = reinterpret_cast<float*>(smem + LY::XCH);   // [2][QM]
+      constexpr int HK = QKT / 2;          // key columns of a half
+      if (q < nsw) {
+        for (int t = 0; t < T; ++t) {
+          const int sb_i = t % LY::NSB;
+          const int st = t % NS;
+          uint8_t* sb = smem + st * LY::STAGE;
+          const bool blk = do_blk && t == n;
+          const int nk = blk ? KBR : QKT;          // score columns of this tile
+          // The two warps of a row pair decide an abort together (from both
+          // votes, read after the first exchange barrier), so neither is left
+          // waiting at a barrier the other no longer reaches.
+          const bool okw =
+              __all_sync(0xffffffffu, mbar_wait(&s_full[sb_i], (uint32_t)(t / LY::NSB) & 1u, Q_WAIT_NS)) &&
+              !*abort_flag;
+          if (lane == 0) xvote[grp * 4 + q] = okw ? 1 : 0;
           tc_fence_after();
-          if (okp) {
-#pragma unroll 1
-            for (int c = 0; c < D / 16; ++c) {
-              float o[16];
-              tq_ld16(lane_base + ocol + c * 16, o);
-              tq_wait_ld();
-              uint32_t w[16];
+          const uint32_t srow = lane_base + (uint32_t)(sb_i * QKT);
+          // keys 0..lim of this tile are visible to this row (raw scores; the
+          // scale is positive, so it is applied with the exponent).  Padding
+          // rows (r >= NR) give rows of P and O that nothing reads, so they
+          // decide neither the masking nor a rescale.
+          const int lim = blk ? blim : min(QKT, C - (t_begin + t) * QKT) - 1;
+          float x[HK];
 #pragma unroll
-              for (int k = 0; k < 16; ++k) w[k] = __float_as_uint(o[k] * alpha);
-              tq_st16(lane_base + ocol + c * 16, w);
+          for (int c = 0; c < HK / 16; ++c) {
+            if (okw && kc0 + c * 16 < nk) {
+              tq_ld16(srow + kc0 + c * 16, &x[c * 16]);
+            } else {
+#pragma unroll
+              for (int k = 0; k < 16; ++k) x[c * 16 + k] = -INFINITY;
             }
-          } else if (lane == 0) {
-            set_err(p.err, ERR_TIMEOUT);
           }
-        }
-        // P = 2^(score * scale - m_ref) in bf16, two keys per TMEM column, over
-        // this half's scores (masked keys give exactly 0)
-        const float nb = (mref == -INFINITY) ? 0.f : -mref;
-        float l4[4] = {0.f, 0.f, 0.f, 0.f};
-        auto exp_store = [&](float (&x)[32], int k0) {
-          uint32_t pk[16];
+          tq_wait_ld();
+          if (__any_sync(0xffffffffu, rvalid && lim < kc0 + HK - 1)) {
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
+            for (int k = 0; k < HK; ++k) x[k] = (kc0 + k <= lim) ? x[k] : -INFINITY;
+          }
+          float m4[4] = {x[0], x[1], x[2], x[3]};
+#pragma unroll
+          for (int k = 4; k < HK; ++k) m4[k & 3] = fmaxf(m4[k & 3], x[k]);
+          const float mh = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+          // the row's maximum over both halves (both threads have read their
+          // scores by the first barrier, so P may then overwrite them; the
+          // second barrier lets the buffer be rewritten at the next tile)
+          xch[grp * QM + r] = mh;
+          named_bar_sync(1 + q, 64);
+          const float mx = fmaxf(mh, xch[(grp ^ 1) * QM + r]) * sc;
+          const bool ok2 = xvote[q] != 0 && xvote[4 + q] != 0;
+          named_bar_sync(1 + q, 64);
+          if (!ok2) {
+            if (lane == 0) {
+              set_err(p.err, ERR_TIMEOUT);
+              *abort_flag = 1;
+            }
+            break;
+          }
+          // move the reference only when a score exceeds it by 2^8 (the first
+          // tile always sets it: m_ref starts at -inf)
+          const bool up = rvalid && mx > mref + Q_LAZY;
+          float alpha = 1.f;
+          if (up) {
+            alpha = (mref == -INFINITY) ? 0.f : exp2_approx(mref - mx);
+            mref = mx;
+            l *= alpha;
+          }
+          if (__any_sync(0xffffffffu, up && t > 0)) {
+            // O holds tiles 0..t-1: wait for the last of them, then scale this
+            // group's half of the row
+            const bool okp =
+                __all_sync(0xffffffffu, mbar_wait(&pv_done[0], (uint32_t)(t - 1) & 1u, Q_WAIT_NS));
+            tc_fence_after();
+            if (okp) {
+#pragma unroll 1
+              for (int c = 0; c < D / 32; ++c) {
+                float o[16];
+                tq_ld16(lane_base + ocol + c * 16, o);
+                tq_wait_ld();
+                uint32_t w[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) w[k] = __float_as_uint(o[k] * alpha);
+                tq_st16(lane_base + ocol + c * 16, w);
+              }
+            } else if (lane == 0) {
+              set_err(p.err, ERR_TIMEOUT);
+            }
+          }
+          // P = 2^(score * scale - m_ref) in bf16, two keys per TMEM column, in
+          // this half's columns of the score buffer (masked keys give exactly 0)
+          const float nb = (mref == -INFINITY) ? 0.f : -mref;
+          float l4[4] = {0.f, 0.f, 0.f, 0.f};
+          uint32_t pk[HK / 2];
+#pragma unroll
+          for (int k = 0; k < HK / 2; ++k) {
             const float p0 = exp2_approx(fmaf(x[2 * k], sc, nb));
             const float p1 = exp2_approx(fmaf(x[2 * k + 1], sc, nb));
             l4[k & 3] += p0 + p1;
             pk[k] = pack_bf16(p0, p1);
           }
-          tq_st16(srow + k0 / 2, pk);
-        };
-        exp_store(x0, 0);
-        exp_store(x1, 32);
-        l += (l4[0] + l4[1]) + (l4[2] + l4[3]);
-        // V rows of keys outside the context (or past the block) may hold
-        // stale bytes: the half's group zeroes them so that their zero weights
-        // contribute 0 (V lands separately from K: wait for it first).
-        const int vr = blk ? p.R : min(QKT / 2, max(0, left));
-        if (vr < nk) {
-          const int st = t % NS;
-          if (__all_sync(0xffffffffu, mbar_wait(&full_v[st], (uint32_t)(t / NS) & 1u, Q_WAIT_NS))) {
-            uint8_t* vb = smem + st * LY::STAGE + LY::KVB + kc0 * QROWB;
-            const int vhalf = (blk ? KBR : QKT) * QROWB;
-            for (int e = r; e < (nk - vr) * H * 8; e += nsw * 32) {
-              const int row = vr + e / (H * 8), rem = e % (H * 8);
-              *reinterpret_cast<uint4*>(vb + (rem / 8) * vhalf + row * QROWB + (rem % 8) * 16) =
-                  make_uint4(0u, 0u, 0u, 0u);
+          l += (l4[0] + l4[1]) + (l4[2] + l4[3]);
+#pragma unroll
+          for (int c = 0; c < HK / 32; ++c)
+            if (kc0 + c * 32 < nk) tq_st16(srow + kc0 / 2 + c * 16, &pk[c * 16]);
+          // V rows of keys outside the context (or past the block) may hold
+          // stale bytes: group 0 zeroes them so that their zero weights
+          // contribute 0 (V lands separately from K: wait for it first).
+          if (grp == 0) {
+            const int vr = blk ? p.R : min(QKT, C - (t_begin + t) * QKT);
+            if (vr < nk &&
+                __all_sync(0xffffffffu, mbar_wait(&full_v[st], (uint32_t)(t / NS) & 1u, Q_WAIT_NS))) {
+              uint8_t* vb = sb + LY::KVB;
+              const int vhalf = nk * QROWB;
+              for (int e = r; e < (nk - vr) * H * 8; e += nsw * 32) {
+                const int row = vr + e / (H * 8), rem = e % (H * 8);
+                *reinterpret_cast<uint4*>(vb + (rem / 8) * vhalf + row * QROWB + (rem % 8) * 16) =
+                    make_uint4(0u, 0u, 0u, 0u);
+              }
+              fence_proxy_async_smem();
             }
-            fence_proxy_async_smem();
+          }
+          tq_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&p_full[2 * sb_i]);
+        }
+        if (T > 0 && !*abort_flag) {
+          const bool okp =
+              __all_sync(0xffffffffu, mbar_wait(&pv_done[0], (uint32_t)(T - 1) & 1u, Q_WAIT_NS));
+          if (!okp && lane == 0) {
+            set_err(p.err, ERR_TIMEOUT);
+            *abort_flag = 1;
           }
         }
+        tc_fence_after();
+      }
+      // the row's sum over both halves (the exchange buffer is free: every
+      // tile's second barrier has passed)
+      if (q < nsw) {
+        xch[grp * QM + r] = l;
+        named_bar_sync(1 + q, 64);
+        l += xch[(grp ^ 1) * QM + r];
+      }
+    } else {
+      const int T_mine = grp ? n : T;      // the block tile's keys are all in half 0
+      if (q < nsw) {
+        for (int t = 0; t < T_mine; ++t) {
+          const bool blk = do_blk && t == n;
+          const int nk = blk ? KBR : QKT / 2;      // score columns of this half
+          if (!__all_sync(0xffffffffu, mbar_wait(&s_full[t & 1], (uint32_t)(t >> 1) & 1u, Q_WAIT_NS)) || *abort_flag) {
+            if (lane == 0) {
+              set_err(p.err, ERR_TIMEOUT);
+              *abort_flag = 1;
+            }
+            break;
+          }
+          tc_fence_after();
+          const uint32_t srow = lane_base + (uint32_t)((t & 1) * QKT + kc0);
+          // keys 0..lim of this half are visible to this row (raw scores; the
+          // scale is positive, so it is applied with the exponent).  Padding
+          // rows (r >= NR) give rows of P and O that nothing reads, so they
+          // decide neither the masking nor a rescale.  A block tile has 16 to 64
+          // score columns; the rest of the half holds an earlier tile's.
+          const int left = C - (t_begin + t) * QKT - kc0;      // context keys from here on
+          const int lim = blk ? blim : min(QKT / 2, left) - 1;
+          float x0[32], x1[32];
+          tq_ld32(srow, x0);
+          tq_ld32(srow + 32, x1);
+          tq_wait_ld32(x0);
+          tq_wait_ld32(x1);
+          if (__any_sync(0xffffffffu, rvalid && lim < QKT / 2 - 1) || blk) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) {
+              x0[k] = k <= lim ? x0[k] : -INFINITY;
+              x1[k] = 32 + k <= lim ? x1[k] : -INFINITY;
+            }
+          }
+          float m4[4] = {x0[0], x0[1], x0[2], x0[3]};
+#pragma unroll
+          for (int k = 4; k < 32; ++k) m4[k & 3] = fmaxf(m4[k & 3], x0[k]);
+#pragma unroll
+          for (int k = 0; k < 32; ++k) m4[k & 3] = fmaxf(m4[k & 3], x1[k]);
+          const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * sc;
+          // move the reference only when a score exceeds it by 2^8 (the first
+          // tile always sets it: m_ref starts at -inf)
+          const bool up = rvalid && mx > mref + Q_LAZY;
+          float alpha = 1.f;
+          if (up) {
+            alpha = (mref == -INFINITY) ? 0.f : exp2_approx(mref - mx);
+            mref = mx;
+            l *= alpha;
+          }
+          if (__any_sync(0xffffffffu, up && t > 0)) {
+            // O_h holds tiles 0..t-1: wait for the last of them, then scale the row
+            const bool okp =
+                __all_sync(0xffffffffu, mbar_wait(&pv_done[grp], (uint32_t)(t - 1) & 1u, Q_WAIT_NS));
+            tc_fence_after();
+            if (okp) {
+#pragma unroll 1
+              for (int c = 0; c < D / 16; ++c) {
+                float o[16];
+                tq_ld16(lane_base + ocol + c * 16, o);
+                tq_wait_ld();
+                uint32_t w[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) w[k] = __float_as_uint(o[k] * alpha);
+                tq_st16(lane_base + ocol + c * 16, w);
+              }
+            } else if (lane == 0) {
+              set_err(p.err, ERR_TIMEOUT);
+            }
+          }
+          // P = 2^(score * scale - m_ref) in bf16, two keys per TMEM column, over
+          // this half's scores (masked keys give exactly 0)
+          const float nb = (mref == -INFINITY) ? 0.f : -mref;
+          float l4[4] = {0.f, 0.f, 0.f, 0.f};
+          auto exp_store = [&](float (&x)[32], int k0) {
+            uint32_t pk[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+              const float p0 = exp2_approx(fmaf(x[2 * k], sc, nb));
+              const float p1 = exp2_approx(fmaf(x[2 * k + 1], sc, nb));
+              l4[k & 3] += p0 + p1;
+              pk[k] = pack_bf16(p0, p1);
+            }
+            tq_st16(srow + k0 / 2, pk);
+          };
+          exp_store(x0, 0);
+          exp_store(x1, 32);
+          l += (l4[0] + l4[1]) + (l4[2] + l4[3]);
+          // V rows of keys outside the context (or past the block) may hold
+          // stale bytes: the half's group zeroes them so that their zero weights
+          // contribute 0 (V lands separately from K: wait for it first).
+          const int vr = blk ? p.R : min(QKT / 2, max(0, left));
+          if (vr < nk) {
+            const int st = t % NS;
+            if (__all_sync(0xffffffffu, mbar_wait(&full_v[st], (uint32_t)(t / NS) & 1u, Q_WAIT_NS))) {
+              uint8_t* vb = smem + st * LY::STAGE + LY::KVB + kc0 * QROWB;
+              const int vhalf = (blk ? KBR : QKT) * QROWB;
+              for (int e = r; e < (nk - vr) * H * 8; e += nsw * 32) {
+                const int row = vr + e / (H * 8), rem = e % (H * 8);
+                *reinterpret_cast<uint4*>(vb + (rem / 8) * vhalf + row * QROWB + (rem % 8) * 16) =
+                    make_uint4(0u, 0u, 0u, 0u);
+              }
+              fence_proxy_async_smem();
+            }
+          }
+          tq_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&p_full[2 * (t & 1) + grp]);
+        }
+        if (T_mine > 0 && !*abort_flag) {
+          const bool okp =
+              __all_sync(0xffffffffu, mbar_wait(&pv_done[grp], (uint32_t)(T_mine - 1) & 1u, Q_WAIT_NS));
+          if (!okp && lane == 0) {
+            set_err(p.err, ERR_TIMEOUT);
+            *abort_flag = 1;
+          }
+        }
+        // (m_ref, l) for the row's other half, through score columns that are free: P takes the
+        // first 32 of a half, and this half's last products are done.
+        tq_st2(lane_base + (uint32_t)(kc0 + 32), mref, l);
         tq_wait_st();
         tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&p_full[2 * (t & 1) + grp]);
       }
-      if (T_mine > 0 && !*abort_flag) {
-        const bool okp =
-            __all_sync(0xffffffffu, mbar_wait(&pv_done[grp], (uint32_t)(T_mine - 1) & 1u, Q_WAIT_NS));
-        if (!okp && lane == 0) {
-          set_err(p.err, ERR_TIMEOUT);
-          *abort_flag = 1;
-        }
-      }
-      tc_fence_before();
     }
   }
   __syncthreads();
   tc_fence_after();
-  // Every MMA is done: the query rows' place takes the (m_ref, l) of the row halves.
-  float2* ml = reinterpret_cast<float2*>(qs);                // [2 halves][QM]
-  if (warp >= Q_SOFT0) ml[tid - Q_SOFT0 * 32] = make_float2(mref, l);
-  __syncthreads();
-
+  const int rpo = (NR + S - 1) / S;
+  if (S > 1) {                           // the ring is idle from here on
+    if (tid == 0) mbar_arrive_expect_tx(recv_bar, (uint32_t)(S * rpo * LY::ROWP));
+    cluster_arrive_relaxed();
+  }
   // ---------------------------------------------------------------- output
   // The ring is idle from here on.  Unsplit, every softmax thread writes its
   // normalised row; split, it writes its partial row (O, m_ref, l) and the
   // cluster's CTAs reduce-scatter them (owner o finishes rows
   // [o * rpo, (o + 1) * rpo)).
   const bool have = T > 0 && !*abort_flag;
-  const int rpo = (NR + S - 1) / S;
-  if (S > 1) {
-    if (tid == 0) mbar_arrive_expect_tx(recv_bar, (uint32_t)(S * rpo * LY::ROWP));
-    cluster_arrive_relaxed();
-  }
   float* part = reinterpret_cast<float*>(smem + LY::PART);
   if (warp >= Q_SOFT0 && ((warp - Q_SOFT0) & 3) < nsw) {
     // The two halves of a row are put together: common maximum, weighted sums.
     // Each group writes half of the row's columns.
     const int sw = warp - Q_SOFT0, grp = sw >> 2, q = sw & 3, r = q * 32 + lane;
     const bool rvalid = r < NR;
-    const int c0 = grp * (D / 32);       // first 16-column chunk of this group's half
+    const int c0 = grp * (D / 64);       // first 32-column chunk of this group's half
     const uint32_t orow = tmem_base + ((uint32_t)(q * 32) << 16) + LY::OCOL;
-    const float2 h0 = ml[r], h1 = ml[QM + r];
-    mref = fmaxf(h0.x, h1.x);
-    const float w0_ = (h0.x == -INFINITY) ? 0.f : exp2_approx(h0.x - mref);
-    const float w1_ = (h1.x == -INFINITY) ? 0.f : exp2_approx(h1.x - mref);
-    l = h0.y * w0_ + h1.y * w1_;
-    const bool have1 = have && n > 0;    // half 1 holds cache tiles only
-    auto load_o = [&](int c, float (&o)[16]) {
-      float o1[16];
+    float w0_ = 1.f, w1_ = 0.f;
+    if constexpr (!SWAP) {
+      float mo, lo;
+      tq_ld2(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)((grp ^ 1) * 64 + 32), mo, lo);
+      const float mm = fmaxf(mref, mo);
+      const float wm = (mref == -INFINITY) ? 0.f : exp2_approx(mref - mm);   // this half's weight
+      const float wo = (mo == -INFINITY) ? 0.f : exp2_approx(mo - mm);
+      mref = mm;
+      l = grp ? lo * wo + l * wm : l * wm + lo * wo;
+      w0_ = grp ? wo : wm;
+      w1_ = grp ? wm : wo;
+    }
+    const bool have1 = !SWAP && have && n > 0;    // half 1 holds cache tiles only
+    // 32 columns at a time, from both accumulators
+    auto load_o = [&](int c, float (&o)[32]) {
+      float o1[32];
       if (have) {
-        tq_ld16(orow + c * 16, o);
-        if (have1) tq_ld16(orow + D + c * 16, o1);
-        tq_wait_ld();
+        tq_ld32(orow + c * 32, o);
+        if (have1) tq_ld32(orow + D + c * 32, o1);
+        tq_wait_ld32(o);
+        if (have1) tq_wait_ld32(o1);
       }
 #pragma unroll
-      for (int i = 0; i < 16; ++i) o[i] = have ? (have1 ? o[i] * w0_ + o1[i] * w1_ : o[i] * w0_) : 0.f;
+      for (int i = 0; i < 32; ++i)
+        o[i] = !have ? 0.f : SWAP ? o[i] : have1 ? o[i] * w0_ + o1[i] * w1_ : o[i] * w0_;
     };
     if (S == 1) {
       const int j = j0 + (rvalid ? r / p.G : 0), g = rvalid ? r % p.G : 0;
       __nv_bfloat16* dst = p.out + (((size_t)b * p.R + j) * p.Hq + (size_t)kvh * p.G + g) * D;
       const float inv = (have && l > 0.f) ? 1.f / l : 0.f;
-#pragma unroll 1
-      for (int c = c0; c < c0 + D / 32; ++c) {
-        float o[16];
+#pragma unroll
+      for (int c = c0; c < c0 + D / 64; ++c) {
+        float o[32];
         load_o(c, o);
         if (rvalid) {
-          uint4 w0, w1;
-          w0.x = pack_bf16(o[0] * inv, o[1] * inv);
-          w0.y = pack_bf16(o[2] * inv, o[3] * inv);
-          w0.z = pack_bf16(o[4] * inv, o[5] * inv);
-          w0.w = pack_bf16(o[6] * inv, o[7] * inv);
-          w1.x = pack_bf16(o[8] * inv, o[9] * inv);
-          w1.y = pack_bf16(o[10] * inv, o[11] * inv);
-          w1.z = pack_bf16(o[12] * inv, o[13] * inv);
-          w1.w = pack_bf16(o[14] * inv, o[15] * inv);
-          *reinterpret_cast<uint4*>(dst + c * 16) = w0;
-          *reinterpret_cast<uint4*>(dst + c * 16 + 8) = w1;
+#pragma unroll
+          for (int i = 0; i < 32; i += 8) {
+            uint4 w;
+            w.x = pack_bf16(o[i] * inv, o[i + 1] * inv);
+            w.y = pack_bf16(o[i + 2] * inv, o[i + 3] * inv);
+            w.z = pack_bf16(o[i + 4] * inv, o[i + 5] * inv);
+            w.w = pack_bf16(o[i + 6] * inv, o[i + 7] * inv);
+            *reinterpret_cast<uint4*>(dst + c * 32 + i) = w;
+          }
         }
       }
     } else {
       float* prow = part + r * PD;
-#pragma unroll 1
-      for (int c = c0; c < c0 + D / 32; ++c) {
-        float o[16];
+#pragma unroll
+      for (int c = c0; c < c0 + D / 64; ++c) {
+        float o[32];
         load_o(c, o);
         if (rvalid) {
 #pragma unroll
-          for (int i = 0; i < 16; i += 4)
-            *reinterpret_cast<float4*>(prow + c * 16 + i) = make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
+          for (int i = 0; i < 32; i += 4)
+            *reinterpret_cast<float4*>(prow + c * 32 + i) = make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
         }
       }
       if (rvalid && grp == 0) {
@@ -727,25 +982,25 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
 }
 
 // At least 118 KB, so that two CTAs (each wants all of TMEM) never share an SM.
-template <int D>
+template <int D, bool SWAP>
 size_t tcq_smem_bytes() {
-  const size_t need = (size_t)TcqLayout<D>::TOTAL + 1024;
+  const size_t need = (size_t)TcqLayout<D, SWAP>::TOTAL + 1024;
   return need > 118 * 1024 ? need : 118 * 1024;
 }
 
 // Limits already set on each instantiation of the kernel.
-template <int D>
+template <int D, bool SWAP>
 KernelLimits& tcq_limits() {
   static KernelLimits lim;
   return lim;
 }
 
-template <int D>
+template <int D, bool SWAP>
 cudaError_t launch_tcq_t(const CUtensorMap* maps, const TcqParams& p, int S, int B, int Hkv, int RG,
                          cudaStream_t stream) {
-  const size_t smem = tcq_smem_bytes<D>();
-  auto kern = verify_attn_tcq_kernel<D>;
-  const cudaError_t e = ensure_kernel_limits((const void*)kern, tcq_limits<D>(), smem, true);
+  const size_t smem = tcq_smem_bytes<D, SWAP>();
+  auto kern = verify_attn_tcq_kernel<D, SWAP>;
+  const cudaError_t e = ensure_kernel_limits((const void*)kern, tcq_limits<D, SWAP>(), smem, true);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(S, Hkv * RG, B);
@@ -764,11 +1019,11 @@ cudaError_t launch_tcq_t(const CUtensorMap* maps, const TcqParams& p, int S, int
   return cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], maps[3], maps[4], p);
 }
 
-template <int D>
+template <int D, bool SWAP>
 int max_cluster_tcq_t(int S, int Hkv, int B, int RG) {
-  const size_t smem = tcq_smem_bytes<D>();
-  auto kern = verify_attn_tcq_kernel<D>;
-  if (ensure_kernel_limits((const void*)kern, tcq_limits<D>(), smem, true) != cudaSuccess) {
+  const size_t smem = tcq_smem_bytes<D, SWAP>();
+  auto kern = verify_attn_tcq_kernel<D, SWAP>;
+  if (ensure_kernel_limits((const void*)kern, tcq_limits<D, SWAP>(), smem, true) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -796,8 +1051,8 @@ int max_cluster_tcq_t(int S, int Hkv, int B, int RG) {
 bool tcq_attn_supported(int D, int G) { return (D == 64 || D == 128) && G >= 1 && G <= QM; }
 
 int attn_tcq_max_active_clusters(int D, int S, int Hkv, int B, int RG) {
-  if (D == 128) return max_cluster_tcq_t<128>(S, Hkv, B, RG);
-  if (D == 64) return max_cluster_tcq_t<64>(S, Hkv, B, RG);
+  if (D == 128) return max_cluster_tcq_t<128, false>(S, Hkv, B, RG);
+  if (D == 64) return max_cluster_tcq_t<64, false>(S, Hkv, B, RG);
   return 0;
 }
 
@@ -848,8 +1103,17 @@ cudaError_t launch_verify_attn_tcq(const AttnArgs& a, const AttnPlan& pl, int* e
   p.kv_stable = a.kv_stable;
   p.block_full = a.block_full;
   p.err = err;
-  if (a.D == 128) return launch_tcq_t<128>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream);
-  if (a.D == 64) return launch_tcq_t<64>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream);
+  // Eight or more CTAs per cluster (batch 1) have two or three tiles each, where the halves' own
+  // accumulators cost more at the end than the swaps on the way: 10.05 us per layer against 9.79
+  // (K = 15) and 11.2 against 10.85 (K = 25); from batch 2 on (longer runs of tiles) they gain, 12.40
+  // against 12.47 and, at batch 4, 18.9 against 19.2.
+  const bool swap = pl.cluster >= 8;
+  if (a.D == 128)
+    return swap ? launch_tcq_t<128, true>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream)
+                : launch_tcq_t<128, false>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream);
+  if (a.D == 64)
+    return swap ? launch_tcq_t<64, true>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream)
+                : launch_tcq_t<64, false>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream);
   return cudaErrorInvalidValue;
 }
 
