@@ -91,7 +91,7 @@ class BlockPrefill:
         step = self.rows // chunk
         self.block_table = self.table2[::step].contiguous()
         self.block_start = self.start[::step].contiguous()
-        # chunk-padded projections [L, B, nck * chunk, H, D], made by the first load()
+        # chunk-padded projections [L, B, nck * chunk, H, D], made when first used
         self.qp = self.kp = self.vp = self.outp = None
 
     def _check(self, q, k, v) -> None:
@@ -99,21 +99,29 @@ class BlockPrefill:
         if tuple(q.shape) != (L, B, C, self.Hq, self.D) or tuple(k.shape) != (L, B, C, self.Hkv, self.D):
             raise ValueError("q / k / v must be [L, B, C, H, D] with the prefill's shape")
 
-    def load(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> None:
-        """q [L, B, C, Hq, D], k / v [L, B, C, Hkv, D] (bf16): the context's
-        per-layer projections, placed into the chunk-padded buffers."""
-        self._check(q, k, v)
+    def _padded(self) -> None:
         if self.qp is None:
             padded = lambda heads: torch.zeros((self.L, self.B, self.nck * self.chunk, heads, self.D),
                                                dtype=torch.bfloat16, device=self.k_pages.device)
             self.qp, self.kp, self.vp = padded(self.Hq), padded(self.Hkv), padded(self.Hkv)
             self.outp = torch.empty_like(self.qp)
+
+    def load(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> None:
+        """q [L, B, C, Hq, D], k / v [L, B, C, Hkv, D] (bf16): the context's
+        per-layer projections, placed into the chunk-padded buffers."""
+        self._check(q, k, v)
+        self._padded()
+        # v may have more rows than the context, or broadcast: then chunk by chunk
+        n = max(1, self.C) if v.shape == k.shape else self.chunk
         for dst, src in ((self.qp, q), (self.kp, k), (self.vp, v)):
-            dst[:, :, :self.C].copy_(src)
+            for c0 in range(0, self.C, n):
+                c1 = min(self.C, c0 + n)
+                dst[:, :, c0:c1].copy_(src[:, :, c0:c1])
 
     def step(self) -> None:
         """The prefill itself, from the loaded buffers: one commit, then one
         attention launch per layer (all launches, no host synchronisation)."""
+        self._padded()
         self._launch(self.qp, self.kp, self.vp, self.outp)
 
     def _launch(self, q, k, v, out) -> None:
@@ -135,11 +143,13 @@ class BlockPrefill:
     def run(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> torch.Tensor:
         """Commits the context's K/V into the cache and returns the attention
         output [L, B, C, Hq, D].  A context of whole chunks is read and written
-        where it lies; a ragged one goes through the padded buffers."""
+        where it lies; a ragged one, and projections of another device, type or
+        layout, go through the padded buffers."""
         self._check(q, k, v)
-        out = torch.empty_like(q, memory_format=torch.contiguous_format)
-        if self.C == self.nck * self.chunk and all(
-                t.is_contiguous() and t.dtype == torch.bfloat16 and t.data_ptr() % 16 == 0 for t in (q, k, v)):
+        out = torch.empty_like(q)
+        if self.C == self.nck * self.chunk and v.shape == k.shape and all(
+                t.device == self.k_pages.device and t.is_contiguous() and t.dtype == torch.bfloat16
+                and t.data_ptr() % 16 == 0 for t in (q, k, v)):
             self._launch(q, k, v, out)
         else:
             self.load(q, k, v)

@@ -76,3 +76,34 @@ def test_prefill_then_region_matches_dense_hybrid_attention(method, L, B, T, Hq,
     for b in range(B):
         t = np.arange(T)
         np.testing.assert_array_equal(kp[:, table[b, t // 16], :, t % 16].transpose(1, 0, 2, 3), kb[:, b])
+
+
+@pytest.mark.parametrize("form", ["host", "float32", "strided", "long_v", "shared_v"])
+def test_block_prefill_takes_every_form_of_the_projections(form):
+    """Whole-chunk contexts whose projections cannot be read where they lie give
+    what the in-place path gives for the same values, bit for bit."""
+    L, B, T, Hq, Hkv, D = 2, 2, 96, 4, 2, 64
+    rng = np.random.default_rng(96)
+    q, k, v = _bf16(rng, (L, B, T, Hq, D)), _bf16(rng, (L, B, T, Hkv, D)), _bf16(rng, (L, B, T, Hkv, D))
+    if form == "shared_v":
+        v = v[:1].expand(L, B, T, Hkv, D).contiguous()
+    plain = BlockPrefill(L, B, T, Hq, Hkv, D)
+    ref = plain.run(q, k, v)
+    if form == "host":
+        q2, k2, v2 = q.cpu(), k.cpu(), v.cpu()
+    elif form == "float32":
+        q2, k2, v2 = q.float(), k.float(), v.float()
+    elif form == "strided":
+        q2, k2, v2 = (t.transpose(1, 2).contiguous().transpose(1, 2) for t in (q, k, v))
+    elif form == "long_v":
+        q2, k2, v2 = q, k, torch.cat([v, v[:, :, :5]], dim=2)
+    else:
+        q2, k2, v2 = q, k, v[:1]
+    other = BlockPrefill(L, B, T, Hq, Hkv, D)
+    other.step()                         # without a load: zero projections
+    out = other.run(q2, k2, v2)
+    torch.cuda.synchronize()
+    assert C.get_device_error() == 0
+    assert out.device == q2.device and out.dtype == q2.dtype and out.stride() == torch.empty_like(q2).stride()
+    assert torch.equal(out.to("cuda", torch.bfloat16), ref)
+    assert torch.equal(other.k_pages, plain.k_pages) and torch.equal(other.v_pages, plain.v_pages)
