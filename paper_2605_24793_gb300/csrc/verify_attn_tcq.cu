@@ -282,8 +282,8 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
           tma_prefetch_l2_3d((lane & 1) ? (const void*)&map_vp : (const void*)&map_kp, 0,
                              (pg * p.Hkv + kvh) * QPAGE, h);
     }
-    // the block K/V comes from the previous kernel; the other producers
-    // read only the (stable) cache
+    // the block K/V comes from the previous kernel: warp 0, which loads its K, waits
+    // here, warp 2 before it loads its V; warp 1 reads only the (stable) cache
     if (p.kv_stable && pw == 0) griddep_wait();
     for (int t = pre; t < n && ok; ++t) {
       if (!wait_slot(t)) {
@@ -295,6 +295,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     }
     if (ok && do_blk) {
       const int t = n;
+      if (p.kv_stable && pw == 2) griddep_wait();
       if (wait_slot(t)) {
         const int st = t % NS;
         uint8_t* sb = smem + st * LY::STAGE;

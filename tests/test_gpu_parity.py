@@ -893,3 +893,40 @@ def test_lmhead_sampling_noise_only_at_huge_temperature():
     clear = _key_margin(keys) >= 1e-3
     assert clear.sum() >= M - 2
     assert np.array_equal(smp.cpu().numpy()[clear], np.argmax(keys, axis=1)[clear])
+
+
+@pytest.mark.parametrize("R,Hkv,G", [(40, 2, 1), (48, 1, 1), (20, 2, 4), (53, 1, 4)])
+@pytest.mark.parametrize("ctx2", [0, 100, 300])
+def test_verify_attn_stable_cache_waits_for_the_block(R, Hkv, G, ctx2):
+    """With the stable-cache promise the block's own K/V may still come from the
+    launch before: a long attention whose output is the short one's block keys
+    and values, back to back, gives what it gives with a synchronisation between."""
+    import torch
+    D, P = 128, 16
+    g = torch.Generator(device="cuda")
+    g.manual_seed(R * 1000 + ctx2)
+    rnd = lambda *sh: torch.randn(*sh, generator=g, device="cuda").to(torch.bfloat16)
+    ctx1 = 16384
+    pages = ctx1 // P
+    kp, vp = rnd(pages, Hkv, P, D), rnd(pages, Hkv, P, D)
+    table = torch.arange(pages, dtype=torch.int32, device="cuda").view(1, pages)
+    c1 = torch.tensor([ctx1], dtype=torch.int32, device="cuda")
+    c2 = torch.tensor([ctx2], dtype=torch.int32, device="cuda")
+    q1, k1, v1 = rnd(1, R, Hkv, D), rnd(1, R, Hkv, D), rnd(1, R, Hkv, D)
+    q2 = rnd(1, R, Hkv * G, D)
+
+    def both(sync):
+        blk = torch.full((1, R, Hkv, D), 3.0, dtype=torch.bfloat16, device="cuda")
+        out = torch.empty_like(q2)
+        torch.cuda.synchronize()
+        C.verify_attn(q1, k1, v1, kp, vp, table, c1, blk, ctx1)
+        if sync:
+            torch.cuda.synchronize()
+        C.verify_attn(q2, blk, blk, kp, vp, table, c2, out, ctx1, kv_stable=True)
+        torch.cuda.synchronize()
+        assert C.get_device_error() == 0
+        return out
+
+    ref = both(True)
+    for _ in range(5):
+        assert torch.equal(both(False), ref)
