@@ -17,8 +17,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libcospec.so")
-SOURCES = ["api.cu", "verify_attn.cu", "verify_attn_tcq.cu", "verify_attn_tcq2.cu", "lmhead.cu", "arbitrate.cu", "rl.cu",
-           "accept_commit.cu", "sps.cu"]
+SOURCES = ["api.cu", "verify_attn.cu", "verify_attn_tcq.cu", "verify_attn_tcq2.cu", "verify_attn_tcp.cu", "lmhead.cu",
+           "arbitrate.cu", "rl.cu", "accept_commit.cu", "sps.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr",
               "-Xcompiler", "-fPIC,-fvisibility=hidden", "-I", os.path.join(ROOT, "include")]

@@ -110,6 +110,22 @@ CS_DEV bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns = 200000
     if (global_timer_ns() - t0 > limit_ns) return false;
   }
 }
+// The same, asleep between polls, for a wait that may be long: a warp that spins (try_wait as well)
+// takes issue slots from the warps of its scheduler.
+CS_DEV bool mbar_wait_idle(uint64_t* bar, uint32_t parity, uint64_t limit_ns = 2000000000ull, uint32_t nap_ns = 20u) {
+  if (mbar_test(bar, parity)) return true;
+  uint64_t t0 = 0;
+#pragma unroll 1
+  for (int i = 0;; ++i) {
+    __nanosleep(nap_ns);
+    if (mbar_test(bar, parity)) return true;
+    if ((i & 63) == 63) {
+      const uint64_t now = global_timer_ns();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > limit_ns) return false;
+    }
+  }
+}
 
 // ---------------------------------------------------------------- TMA
 CS_DEV void tma_prefetch_desc(const void* map) {
@@ -191,6 +207,9 @@ CS_DEV uint32_t dsmem_map(uint32_t local, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
   return r;
+}
+CS_DEV void dsmem_store_u32(uint32_t addr_cluster, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr_cluster), "r"(v) : "memory");
 }
 // Bulk copy of `bytes` (multiple of 16) from this CTA's shared memory to
 // another CTA's shared memory in the cluster; completion is counted on the
@@ -281,6 +300,11 @@ CS_DEV void tma_load_2d_pair(uint32_t dst, const void* map, uint32_t bar_cluster
 // Arrive on a barrier of any CTA of the cluster.
 CS_DEV void mbar_arrive_cluster(uint32_t bar_cluster) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster)
+               : "memory");
+}
+// The same without the release: for what tcgen05 fences order (TMEM).
+CS_DEV void mbar_arrive_cluster_relaxed(uint32_t bar_cluster) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster)
                : "memory");
 }
 
@@ -423,6 +447,85 @@ CS_DEV void umma_commit_on(uint32_t on, uint64_t* bar) {
           smem_u32(bar)),
       "r"(on)
       : "memory");
+}
+
+// The pair forms (see above), issued by a converged warp of the leader.
+CS_DEV void umma_bf16_tmem_a_pair_on(uint32_t on, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+                                     uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(on)
+      : "memory");
+}
+// Four MMAs of 16 along K: operands in 128-byte rows (32 bytes on per MMA); P in TMEM (8 columns
+// on) against an MN-major operand (16 rows of 128 bytes on).
+CS_DEV void umma_bf16_pair_k64_on(uint32_t on, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                  uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q, t;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " setp.eq.b32 t, %4, %4;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n add.s64 a, %1, 2;\n add.s64 b, %2, 2;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n add.s64 a, %1, 4;\n add.s64 b, %2, 4;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n add.s64 a, %1, 6;\n add.s64 b, %2, 6;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, t;\n}\n" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(on)
+      : "memory");
+}
+CS_DEV void umma_bf16_tmem_a_pair_k64_on(uint32_t on, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+                                         uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q, t;\n .reg .b64 b;\n .reg .b32 a;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " setp.eq.b32 t, %4, %4;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n add.s32 a, %1, 8;\n add.s64 b, %2, 128;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n add.s32 a, %1, 16;\n add.s64 b, %2, 256;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n add.s32 a, %1, 24;\n add.s64 b, %2, 384;\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], [a], b, %3, t;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(on)
+      : "memory");
+}
+// Arrives in the two CTAs of `mask` (bits: cluster ranks).
+CS_DEV void umma_commit_pair_on(uint32_t on, uint64_t* bar, uint32_t mask) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n"
+      " @q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}\n" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)mask), "r"(on)
+      : "memory");
+}
+CS_DEV void tma_load_3d_pair(uint32_t dst, const void* map, uint32_t bar_cluster, int x, int y, int z,
+                             uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(dst),
+      "l"(map), "r"(bar_cluster), "r"(x), "r"(y), "r"(z), "l"(policy)
+      : "memory");
+}
+CS_DEV void tma_load_4d_pair(uint32_t dst, const void* map, uint32_t bar_cluster, int x, int y, int z, int w,
+                             uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2], %7;" ::"r"(dst),
+      "l"(map), "r"(bar_cluster), "r"(x), "r"(y), "r"(z), "r"(w), "l"(policy)
+      : "memory");
+}
+
+// Two 32-bit operations in one instruction, each rounded as by itself.
+CS_DEV float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%6, %7};\n"
+      " fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}\n"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+CS_DEV float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
+      " add.rn.f32x2 d, a, b;\n mov.b64 {%0, %1}, d;\n}\n"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
 }
 
 // Programmatic dependent launch: wait until the grids this one depends on

@@ -82,9 +82,11 @@ struct AttnPlan {
   int mt, wk, nrp;        // mma.sync: row tiles, key groups, padded rows
   int nt, jb, jbq, rg;    // tcgen05: row capacity of a row tile (128), block rows per row
                           // tile, block rows of the query box, row groups
-  int two;                // tcgen05: a row group is two row tiles sharing the cache stream
+  int two;                // tcgen05: a row group is two row tiles sharing the cache stream,
+                          // 1: of one CTA, 2: of a CTA pair
   int jg;                 // tcgen05: block rows per row group
   int cluster;            // CTAs per (sequence, KV head, row group): the KV split
+  long long resident;     // tcgen05, CTA pairs: pairs resident at once
   long long units;        // (sequence, KV head, row group) units, one cluster each
   int one_wave;           // small batch: take the largest split whose clusters are
                           // all resident at once (latency-bound)
@@ -99,6 +101,8 @@ cudaError_t launch_verify_attn(const AttnArgs& a, const AttnPlan& plan, int* err
                                cudaStream_t stream);
 cudaError_t launch_verify_attn_tcq2(const AttnArgs& a, const AttnPlan& plan, int* err,
                                     cudaStream_t stream);
+cudaError_t launch_verify_attn_tcp(const AttnArgs& a, const AttnPlan& plan, int* err,
+                                   cudaStream_t stream);
 bool tcq_attn_supported(int D, int G);
 int attn_tcq_max_active_clusters(int D, int S, int Hkv, int B, int RG);
 cudaError_t launch_verify_attn_tcq(const AttnArgs& a, const AttnPlan& plan, int* err,

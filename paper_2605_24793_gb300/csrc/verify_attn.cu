@@ -674,41 +674,49 @@ int variant_mt(int NR) {   // NR <= 64
 }  // namespace
 
 // Row groups and KV split of a tcgen05 launch that is not a small batch: with more than 128 query
-// rows per KV head, groups of 128 (one MMA row tile per CTA) or of 256 (two row tiles sharing a K/V
-// stream, unsplit), and 1 to 16 splits, by the smallest estimated time.  The estimate is a CTA's
-// fixed cost, its merge when split, and its 128-key tiles as measured on GB300 (us; one row tile 7 +
-// 3.5 + 0.94 per tile, two 7.5 + 1.9), put together for equal contexts (whole waves of resident
-// clusters, a further one at 15 % more) and for contexts that average 0.65 of the longest (the longest
-// CTA, or the work spread over the resident clusters), weighted 0.35 to 0.65 since only the
-// longest context is known here.  Against the former rule (128 rows per group, powers of two near one
-// wave of CTAs), us per launch: K = 25 regions (212 rows) at batch 4, 4096 keys 37.8 -> 28.3, batch 8
-// 57.5 -> 40.0, batch 16 83.7 -> 77.6, batch 16 at 2048..4096 keys 66.3 -> 60.5, at 512 keys
-// 23.9 -> 16.3; 208 rows, batch 32 at 2048..8192 keys 184.8 -> 152; K = 7 regions (68 rows) at batch 16,
-// 4096 keys 56 -> 44.
-static AttnPlan plan_tcq(const AttnPlan& base, int B, int R, int Hkv, int max_ctx,
+// rows per KV head, groups of 128 (one MMA row tile per CTA, 1 to 16 splits) or of 256, unsplit (two
+// row tiles sharing a K/V stream in one CTA, or a persistent CTA pair for head dimension 128), by the
+// smallest estimated time.  The estimates are as measured on GB300 (us): a CTA 7 + 0.94 per 128-key
+// tile, 3.5 more when split; two row tiles 7.5 + 1.9 per tile, whole waves of either at 15 % more from
+// the second on; a pair 3 and 4.4 + 0.79 per tile for each of its units.  They are put together for
+// equal contexts (whole waves, whole rounds of units) and for contexts that average 0.65 of the
+// longest (the longest CTA or unit, or the work spread over the resident clusters), weighted 0.35 to
+// 0.65 since only the longest context is known here.  Against the rule before (128 rows per group,
+// powers of two near one wave of CTAs), us per launch: K = 25 regions (212 rows) at batch 4, 4096 keys
+// 37.8 -> 26.6, batch 8 57.5 -> 32.0, batch 16 83.7 -> 60.9, batch 16 at 2048..4096 keys 66.3 -> 48.5, at
+// 512 keys 23.9 -> 15.9; 208 rows, batch 32 at 2048..8192 keys 184.8 -> 133; K = 7 regions (68 rows) at
+// batch 16, 4096 keys 56 -> 44.
+static AttnPlan plan_tcq(const AttnPlan& base, int B, int R, int Hkv, int D, int max_ctx,
                          const ResidentFn& resident) {
   const int tiles = (max_ctx + 127) / 128;
   AttnPlan best = base;
   best.cluster = 1;
   double best_t = -1.0;
-  for (int two = 0; two < (R > base.jb ? 2 : 1); ++two) {
+  for (int two = 0; two < (R <= base.jb ? 1 : D == 128 ? 3 : 2); ++two) {
     AttnPlan pl = base;
     pl.two = two;
-    pl.jg = (two + 1) * base.jb;
+    pl.jg = (two ? 2 : 1) * base.jb;
     pl.rg = (R + pl.jg - 1) / pl.jg;
     pl.units = (long long)B * Hkv * pl.rg;
-    const double fixed = two ? 7.5 : 7.0, merge = 3.5, per_tile = two ? 1.9 : 0.94;
     for (int s = 1; s <= (two ? 1 : 16); ++s) {
       // at least two tiles per CTA; no CTA with more than 256
       if (s > 1 && s * 2 > tiles) break;
       if (s < 16 && (tiles + s - 1) / s > 256) continue;
-      const long long fit = resident(pl, s);
+      const long long fit = resident(pl, two == 2 ? 2 : s);
       if (fit < 1) continue;
-      const double start = fixed + (s > 1 ? merge : 0.0);
-      const double longest = start + per_tile * ((tiles + s - 1) / s);
+      pl.resident = fit;
       const long long waves = (pl.units + fit - 1) / fit;
-      const double equal = waves * longest * (waves > 1 ? 1.15 : 1.0);
-      const double spread = (double)pl.units / fit * (start + per_tile * 0.65 * tiles / s);
+      double equal, longest, spread;
+      if (two == 2) {
+        equal = 3.0 + waves * (4.4 + 0.79 * tiles);
+        longest = 3.0 + (4.4 + 0.79 * tiles);
+        spread = 3.0 + (double)pl.units / fit * (4.4 + 0.79 * 0.65 * tiles);
+      } else {
+        const double per_tile = two ? 1.9 : 0.94, start = two ? 7.5 : s > 1 ? 10.5 : 7.0;
+        longest = start + per_tile * ((tiles + s - 1) / s);
+        equal = waves * longest * (waves > 1 ? 1.15 : 1.0);
+        spread = (double)pl.units / fit * (start + per_tile * 0.65 * tiles / s);
+      }
       const double t = 0.35 * equal + 0.65 * (longest > spread ? longest : spread);
       if (best_t < 0.0 || t < best_t) {
         best_t = t;
@@ -749,14 +757,14 @@ AttnPlan plan_verify_attn(int B, int R, int Hq, int Hkv, int D, int max_ctx, int
     pl.jg = jb;
     pl.rg = (R + jb - 1) / jb;
     pl.nt = 128;
-    if (R > jb) return plan_tcq(pl, B, R, Hkv, max_ctx, resident);
+    if (R > jb) return plan_tcq(pl, B, R, Hkv, D, max_ctx, resident);
     // 128-key tiles, one CTA per SM (a 192 KB stage ring).  A small batch
     // (latency-bound): every cluster resident at once, and down to two tiles
     // per CTA; else by estimate.
     const int tiles_tc = (max_ctx + 127) / 128;
     pl.units = (long long)B * Hkv * pl.rg;
     pl.one_wave = (pl.units * 4 <= num_sms && tiles_tc <= 256) ? 1 : 0;
-    if (!pl.one_wave) return plan_tcq(pl, B, R, Hkv, max_ctx, resident);
+    if (!pl.one_wave) return plan_tcq(pl, B, R, Hkv, D, max_ctx, resident);
     int s = 16;
     while (s > 1 && (s * 2 > tiles_tc || resident(pl, s) < pl.units)) --s;
     pl.cluster = s;
@@ -812,7 +820,9 @@ int attn_max_active_clusters(int D, int mt, int wk, int S, int Hkv, int B, int k
 cudaError_t launch_verify_attn(const AttnArgs& a, const AttnPlan& pl, int* err,
                                cudaStream_t stream) {
   if (pl.kind == 1)
-    return pl.two ? launch_verify_attn_tcq2(a, pl, err, stream) : launch_verify_attn_tcq(a, pl, err, stream);
+    return pl.two == 2 ? launch_verify_attn_tcp(a, pl, err, stream)
+           : pl.two    ? launch_verify_attn_tcq2(a, pl, err, stream)
+                       : launch_verify_attn_tcq(a, pl, err, stream);
   // Pool as {64 columns, rows, half}: a {64, 16, H} box is one page of one
   // head, both 128-byte halves, landing as [half][16 rows][128 B].
   CUtensorMap maps[4];

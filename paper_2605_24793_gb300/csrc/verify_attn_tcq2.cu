@@ -31,9 +31,9 @@
 // make one chain of scores, softmax and P.V (4300-4500 measured, in step or staggered);
 // one row tile per CTA is held to about 1900 cycles per 128 rows by the K/V boxes (2 KB
 // each, about 58 cycles apart in an SM however many warps issue them).
-// Measured (GB300): four layers of a 4096-token causal prefill (32 / 8 heads) 679 us with
-// one row tile per CTA, 570 with two; 208 rows, batch 32 at 2048..8192 keys, 172 -> 152 us
-// per layer; 212 rows, batch 16 at 512 keys, 22.9 -> 16.4.
+// Measured (GB300): 212 rows, batch 16 at 512 keys, 22.9 us per layer with one row tile per
+// CTA, 16.2 with two, 20.4 with CTA pairs (which take head dimension 128 at more keys or
+// units); at 128 keys 10.3 against 16.4 with pairs.
 #include <cuda.h>
 #include <math.h>
 

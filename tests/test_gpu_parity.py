@@ -930,3 +930,66 @@ def test_verify_attn_stable_cache_waits_for_the_block(R, Hkv, G, ctx2):
     ref = both(True)
     for _ in range(5):
         assert torch.equal(both(False), ref)
+
+
+# 200 units of 640 keys and more go to the CTA pairs: row groups whose second CTA has 4, 84 or
+# 128 rows, two row groups, block keys padded to 32 and 64, contexts at every tile edge, more
+# units per cluster than two, a batch above the ranked ones and one of more clusters than fit.
+PAIR_CTX = [0, 1, 15, 16, 17, 63, 64, 65, 127, 128, 129, 191, 192, 255, 256, 257, 383, 384, 511, 512, 513, 639, 640]
+
+
+@pytest.mark.parametrize("full", [False, True], ids=["causal", "full"])
+@pytest.mark.parametrize("B,R,Hq,Hkv", [
+    (100, 33, 8, 2), (100, 53, 8, 2), (100, 64, 8, 2), (100, 17, 16, 2), (100, 64, 16, 2), (420, 33, 4, 1),
+    (420, 33, 32, 8),
+])
+def test_verify_attention_pair_edges(B, R, Hq, Hkv, full):
+    D = 128
+    rng = np.random.default_rng(B + R * 100 + Hq)
+    ctx = [PAIR_CTX[(i * 7) % len(PAIR_CTX)] for i in range(B)]
+    t = _paged_case(rng, B, R, Hq, Hkv, D, ctx, True)
+    assert C.verify_attn_plan(t["q"], t["k_pages"], t["page_table"], max(ctx)) == (C.ATTN_TCGEN05, 1)
+    out = torch.empty_like(t["q"])
+    for b in range(B):                   # the rest of each last page is NaN
+        if ctx[b] % 16:
+            page = int(t["table_np"][b, ctx[b] // 16])
+            t["k_pages"][page, :, ctx[b] % 16:] = float("nan")
+            t["v_pages"][page, :, ctx[b] % 16:] = float("nan")
+    C.verify_attn(t["q"], t["k_blk"], t["v_blk"], t["k_pages"], t["v_pages"], t["page_table"],
+                  t["ctx_len"], out, max(ctx), block_full=full)
+    sub = np.arange(B) if B * Hq <= 1600 else np.sort(rng.permutation(B)[:40])
+    pick = lambda x: host(x[torch.from_numpy(sub).cuda()])
+    ref = O.verify_attention(pick(t["q"]), pick(t["k_blk"]), pick(t["v_blk"]),
+                             np.nan_to_num(host(t["k_pages"])), np.nan_to_num(host(t["v_pages"])),
+                             t["table_np"][sub], t["ctx_np"][sub], 16, **({"block_mask": "full"} if full else {}))
+    assert_close(pick(out), ref, "attention (CTA pairs)")
+    # a second call on other contexts gives the same where the context is the same
+    ctx2 = t["ctx_len"].clone()
+    ctx2[::3] = 0
+    out2 = torch.full_like(out, float("nan"))
+    C.verify_attn(t["q"], t["k_blk"], t["v_blk"], t["k_pages"], t["v_pages"], t["page_table"],
+                  ctx2, out2, max(ctx), block_full=full)
+    keep = torch.arange(B, device="cuda") % 3 != 0
+    assert torch.equal(out2[keep], out[keep])
+    assert not torch.isnan(out2).any()
+    assert C.get_device_error() == 0
+
+
+def test_verify_attention_pair_skips_only_the_bad_sequence():
+    B, R, Hq, Hkv, D = 100, 53, 8, 2, 128
+    rng = np.random.default_rng(53)
+    ctx = [640 - 3 * i for i in range(B)]
+    t = _paged_case(rng, B, R, Hq, Hkv, D, ctx, True)
+    call = lambda c, o: C.verify_attn(t["q"], t["k_blk"], t["v_blk"], t["k_pages"], t["v_pages"],
+                                      t["page_table"], c, o, 640)
+    good, out = torch.empty_like(t["q"]), torch.full_like(t["q"], float("nan"))
+    call(t["ctx_len"], good)
+    assert C.get_device_error() == 0
+    bad = t["ctx_len"].clone()
+    bad[5], bad[70] = -1, t["page_table"].shape[1] * 16 + 1
+    call(bad, out)
+    torch.cuda.synchronize()
+    assert C.get_device_error() == C.DEVERR_CTX
+    skip = torch.zeros(B, dtype=torch.bool, device="cuda")
+    skip[[5, 70]] = True
+    assert torch.equal(out[~skip], good[~skip]) and (out[skip] == 0).all()
