@@ -472,7 +472,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(tempty_leader + (uint32_t)acc * 8u);
+      // (TMEM reads only, which the tcgen05 fences order: a release to the cluster waits for every
+      // store under way; 1024 x 32003, 256 rows: 24.3 -> 23.7 us, 5120 x 151936 264 -> 263)
+      if (lane == 0) mbar_arrive_cluster_relaxed(tempty_leader + (uint32_t)acc * 8u);
     }
     griddep_launch_dependents();
     // the four quarters' statistics of every column merge through the buffers
