@@ -91,8 +91,11 @@ class BlockPrefill:
         step = self.rows // chunk
         self.block_table = self.table2[::step].contiguous()
         self.block_start = self.start[::step].contiguous()
-        # chunk-padded projections [L, B, nck * chunk, H, D], made when first used
+        # chunk-padded projections [L, B, nck * chunk, H, D]; whole chunks need them for inputs
+        # that cannot be read in place only, and have no padding rows to be zero
         self.qp = self.kp = self.vp = self.outp = None
+        if context != self.nck * chunk:
+            self._padded()
 
     def _check(self, q, k, v) -> None:
         L, B, C = self.L, self.B, self.C
