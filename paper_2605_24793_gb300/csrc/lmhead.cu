@@ -25,14 +25,18 @@
 // merges the per-CTA partials.
 //
 // Bound: HBM up to about 200 rows, then the operands' way into the SMs (about 13.5
-// TB/s over the chip) and the tensor pipe.  Measured on GB300, us per call, one CTA
-// per MMA with the butterfly -> this kernel:
-//   Qwen3-8B (d 4096, V 151936)   6 rows 187.3 -> 181.2 (1.02 of the copy peak),
-//     128 rows 200.7 -> 187.9, 256 rows 238.9 -> 205.2
-//   Qwen3-32B (d 5120)            256 rows 289.5 -> 252.7 (0.91 of the copy peak)
-//   Llama-3-8B (V 128256)         384 rows 375.1 -> 302.9, 512 rows 421.5 -> 323.8
-//     (1.66 PFLOP/s)
-//   d 1024, V 32003               256 rows 55.7 -> 24.0, 512 rows 110.7 -> 36.2
+// TB/s over the chip) and the tensor pipe.  The MMAs of a k-block are issued by a
+// converged warp, four to a statement: from one diverged thread an MMA took 100 cycles
+// and several times that beside the epilogue's warps on its scheduler, which held up the
+// mainloop for as long as an epilogue ran (all modes: 128 rows 188 -> 181 us, sampling
+// 207 -> 187.5; 384 rows 346 -> 281).  Measured on GB300, us per call, one CTA per MMA
+// with the butterfly -> this kernel:
+//   Qwen3-8B (d 4096, V 151936)   6 rows 187.3 -> 181 to 184 (the copy peak),
+//     128 rows 200.7 -> 180.1, 256 rows 238.9 -> 196.2
+//   Qwen3-32B (d 5120)            256 rows 289.5 -> 243.4 (0.95 of the copy peak)
+//   Llama-3-8B (V 128256)         384 rows 375.1 -> 244.9, 512 rows 421.5 -> 297.9
+//     (1.81 PFLOP/s)
+//   d 1024, V 32003               256 rows 55.7 -> 22.2, 512 rows 110.7 -> 30.6
 //
 // Statistics are kept as a tuple (m, i, sec, s, t): max logit, its lowest
 // id, second largest logit, s = sum e^(x-m), t = sum e^(x-m) (x-m); then
@@ -327,7 +331,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader)
-    if (lane == 0 && rank == 0) {
+    // (the whole warp walks along; one elected thread acts)
+    if (rank == 0) {
+      const uint32_t on = elect_one();
+      const uint64_t a_desc = smem_desc_sw128(smem_u32(smem + L.a_off));
+      const uint64_t b_desc = smem_desc_sw128(smem_u32(smem + L.b_off));
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -335,40 +343,31 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       for (int tile = tile0; tile < p.num_tiles && ok; tile += tile_step, ++it) {
         const int acc = it & 1;
         const uint32_t aph = (uint32_t)(it >> 1) & 1u;
-        if (!mbar_wait(&tempty[acc], aph ^ 1u, WAIT_NS) || *abort_flag) {
-          ok = false;
-          break;
-        }
+        ok = __all_sync(0xffffffffu, mbar_wait(&tempty[acc], aph ^ 1u, WAIT_NS)) && !*abort_flag;
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * p.n_mma);
         for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&full[stage], phase, WAIT_NS) || *abort_flag) {
-            ok = false;
-            break;
-          }
+          ok = __all_sync(0xffffffffu, mbar_wait(&full[stage], phase, WAIT_NS));
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + L.a_off + (uint32_t)stage * A_BYTES);
-          const uint32_t sb = smem_u32(smem + L.b_off + (uint32_t)stage * b_bytes);
-#pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            umma_bf16_pair(d_tmem, smem_desc_sw128(sa + k * 32), smem_desc_sw128(sb + k * 32), idesc,
-                           (kb | k) != 0 ? 1u : 0u);
-          }
-          umma_commit_pair(&empty[stage]);
+          umma_bf16_pair_k64_on(on, d_tmem, a_desc + (uint64_t)(stage * (A_BYTES >> 4)),
+                                b_desc + (uint64_t)((uint32_t)stage * (b_bytes >> 4)), idesc, kb != 0 ? 1u : 0u);
+          umma_commit_pair_on(on, &empty[stage], 3);
           if (++stage == p.stages) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        umma_commit_pair(&tfull[acc]);
+        umma_commit_pair_on(on, &tfull[acc], 3);
       }
-      if (!ok) {
+      if (!ok && on) {
         set_err(p.err, ERR_TIMEOUT);
         *abort_flag = 1;
       }
-      // every MMA issued by this thread completes before TMEM is released
-      umma_commit_pair(mma_done);
+      // every MMA issued by this warp's thread completes before TMEM is released
+      umma_commit_pair_on(on, mma_done, 3);
       mbar_wait(mma_done, 0, WAIT_NS);
     }
   } else {
