@@ -143,7 +143,10 @@ typedef struct {
 /* The call may start reading ctx_len, page_table and the cached pages before
  * the kernel queued just before it on the stream has finished: set it only
  * when that kernel writes none of them (e.g. between the layers of one
- * round, where only q / k_blk / v_blk come from the previous layer). */
+ * round, where only q / k_blk / v_blk come from the previous layer).  A run of
+ * calls with the flag starts no earlier than the call without it before them,
+ * which has waited for everything queued ahead of itself: a commit, then one
+ * call without the flag, then calls with it read what the commit wrote. */
 #define COSPEC_ATTN_KV_STABLE 1
 
 /* Every block row attends to every block row instead of rows 0..j only: the

@@ -246,7 +246,8 @@ def verify_attn(q, k_blk, v_blk, k_pages, v_pages, page_table, ctx_len, out, max
                 block_full: bool = False) -> torch.Tensor:
     """Verify attention of one layer (Sec. 3.1, Eq. 2).  See include/cospec.h.
     ``kv_stable``: the kernel queued just before writes neither ctx_len, the
-    page table nor the cached pages (COSPEC_ATTN_KV_STABLE).  ``block_full``:
+    page table nor the cached pages (COSPEC_ATTN_KV_STABLE);
+    those before it are waited for by the last call without the flag.  ``block_full``:
     block rows see the whole block (the arbitrator's draft/target region,
     Sec. 3.3; COSPEC_ATTN_BLOCK_FULL)."""
     for t, n in ((q, "q"), (k_blk, "k_blk"), (v_blk, "v_blk"), (k_pages, "k_pages"),

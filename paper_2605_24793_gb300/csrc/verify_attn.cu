@@ -234,14 +234,15 @@ __global__ void __launch_bounds__(MT >= 4 && GEN < 2 ? 192 : MT * WK * 32 + 64,
     fence_barrier_init();
   }
   __syncthreads();
-  // Let the next kernel of the stream start launching right away: its CTAs
-  // take the SMs' free slots and, with the stable-cache promise, stream their
-  // cache tiles while this kernel computes (their own waits keep the order).
-  griddep_launch_dependents();
   // Without the stable-cache promise, wait for the previous kernel before
   // reading anything; with it, only q and the block K/V (read below, after
   // the wait) may come from that kernel, so the cache stream starts now.
   if (!p.kv_stable) griddep_wait();
+  // Then let the next kernel of the stream start launching: its CTAs take the SMs'
+  // free slots and, with the stable-cache promise, stream their cache tiles while this
+  // kernel computes.  Not before the wait: a dependent under the promise reads the
+  // cache at once, and what was queued before this kernel may still be writing it.
+  griddep_launch_dependents();
 
   // Sequences are taken longest context first (blockIdx.z = rank, ties by
   // index), so that the long ones start early and the short ones fill in

@@ -162,8 +162,9 @@ __global__ void __launch_bounds__(TP_THREADS, 1)
     fence_barrier_init();
   }
   if (warp == TP_MMA_WARP) tmem_alloc_pair(tmem_holder, TP_TCOLS);
-  griddep_launch_dependents();
+  // (in this order: a dependent under the stable-cache promise reads the cache at once)
   if (!p.kv_stable) griddep_wait();
+  griddep_launch_dependents();
   // Sequences longest context first (ties to the lower index); a larger batch in index
   // order, from the longer end.
   const bool ranked = p.B <= TP_THREADS;

@@ -185,9 +185,10 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
   // Let the next kernel of the stream start launching; with the stable-cache
-  // promise its CTAs stream their cache tiles while this one computes.
-  griddep_launch_dependents();
+  // promise its CTAs stream their cache tiles while this one computes (so without
+  // the promise only after the wait: what came before may still write the cache).
   if (!p.kv_stable) griddep_wait();
+  griddep_launch_dependents();
 
   // Sequences are taken longest context first (blockIdx.z = rank, ties by
   // index), so that the long ones start early and the short ones fill in

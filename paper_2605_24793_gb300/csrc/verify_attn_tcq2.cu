@@ -151,8 +151,9 @@ __global__ void __launch_bounds__(T2_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
-  griddep_launch_dependents();
+  // (in this order: a dependent under the stable-cache promise reads the cache at once)
   if (!p.kv_stable) griddep_wait();
+  griddep_launch_dependents();
 
   const int b = p.B > RANK_MAX_B ? sequence_in_order(p.ctx_len, p.B, (int)blockIdx.z)
                 : p.B > 1        ? sequence_by_rank(p.ctx_len, p.B, (int)blockIdx.z, seq_slot)

@@ -138,7 +138,8 @@ class BlockPrefill:
         qc, oc = (t.view(L, blocks, rows, self.Hq, self.D) for t in (q, out))
         kc, vc = (t.view(L, blocks, rows, self.Hkv, self.D) for t in (k, v))
         for l in range(L):
-            # layers after the first follow an attention launch, which writes no cache
+            # layers after the first follow an attention launch, which writes no cache, and start
+            # no earlier than the first has waited for the commit
             cs.verify_attn(qc[l], kc[l], vc[l], self.k_pages[l], self.v_pages[l], self.block_table,
                            self.block_start, oc[l], self.max_ctx, kv_stable=l > 0)
         self.ctx_len.fill_(self.C)

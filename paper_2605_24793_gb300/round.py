@@ -127,7 +127,8 @@ class VerifyRound:
         pl = 0 if self.k_pages.shape[0] == 1 else l
         out = self.attn_out[l if self.attn_out.shape[0] > 1 else 0]
         # Layers after the first follow another attention launch, which writes
-        # neither the context lengths, the page table nor the cached pages.
+        # neither the context lengths, the page table nor the cached pages,
+        # and start no earlier than layer 0 has waited for what came before the round.
         return C.verify_attn(self.q[l], self.k_blk[l], self.v_blk[l], self.k_pages[pl],
                              self.v_pages[pl], self.page_table, self.ctx_len, out, self.max_ctx,
                              kv_stable=(l > 0) if kv_stable is None else kv_stable)

@@ -993,3 +993,54 @@ def test_verify_attention_pair_skips_only_the_bad_sequence():
     skip = torch.zeros(B, dtype=torch.bool, device="cuda")
     skip[[5, 70]] = True
     assert torch.equal(out[~skip], good[~skip]) and (out[skip] == 0).all()
+
+
+@pytest.mark.parametrize("batch,k,ctx,layers", [(1, 4, 40, 12), (2, 7, 100, 12), (3, 15, 300, 8)])
+def test_rounds_queued_without_a_restore_read_the_round_before(monkeypatch, batch, k, ctx, layers):
+    """Three rounds on a growing context, captured back to back and replayed, give what the
+    same launches give with a synchronisation after each, bit for bit: the second layer of a round
+    starts early, but not before the commit of the round before is done."""
+    cfg = W.CONFIGS["tiny"].replace(batch=batch, k=k, ctx_lo=ctx, ctx_hi=ctx, layers=layers, mismatch_rate=0.3)
+
+    def new_round():
+        inp = W.make_round_inputs(cfg, device="cuda", extra_tokens=3 * (k + 1))
+        draft = W.synth_drafts(cfg, O.topk_ids(O.lmhead_logits(inp["hidden"].cpu(), inp["w"].cpu()), 8)
+                               .reshape(cfg.batch, cfg.rows, 8))
+        return VerifyRound(inp, draft, max_ctx=ctx + 3 * (k + 1), keep_attn=True)
+
+    def restart(rnd, seed):
+        g = torch.Generator(device="cuda")
+        g.manual_seed(seed)
+        for t in (rnd.k_blk, rnd.v_blk, rnd.q):
+            t.normal_(generator=g)
+        rnd.restore_context()
+
+    def state(rnd):
+        return [t.clone() for t in (rnd.attn_out, rnd.k_pages, rnd.v_pages, rnd.ctx_len, rnd.emitted)]
+
+    rnd, ref = new_round(), new_round()
+    restart(rnd, 0)
+    rnd.run(restore=False)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(3):
+            rnd.run(restore=False)
+    got = []
+    for seed in (1, 2, 3):
+        restart(rnd, seed)
+        graph.replay()
+        got.append(state(rnd))
+    torch.cuda.synchronize()
+    for name in ("verify_attn", "accept_commit"):
+        call = getattr(C, name)
+        monkeypatch.setattr(C, name, lambda *a, _call=call, **kw: (_call(*a, **kw), torch.cuda.synchronize())[0])
+    restart(ref, 0)
+    ref.run(restore=False)
+    for seed, have in zip((1, 2, 3), got):
+        restart(ref, seed)
+        for _ in range(3):
+            ref.run(restore=False)
+        for a, b in zip(have, state(ref)):
+            assert torch.equal(a, b)
+    assert C.get_device_error() == 0

@@ -107,3 +107,46 @@ def test_block_prefill_takes_every_form_of_the_projections(form):
     assert out.device == q2.device and out.dtype == q2.dtype and out.stride() == torch.empty_like(q2).stride()
     assert torch.equal(out.to("cuda", torch.bfloat16), ref)
     assert torch.equal(other.k_pages, plain.k_pages) and torch.equal(other.v_pages, plain.v_pages)
+
+
+def _synchronised(monkeypatch, name):
+    """The binding's call `name`, waited for before it returns."""
+    call = getattr(C, name)
+
+    def synced(*args, **kw):
+        out = call(*args, **kw)
+        torch.cuda.synchronize()
+        return out
+
+    monkeypatch.setattr(C, name, synced)
+
+
+@pytest.mark.parametrize("L,T,Hq,Hkv,D", [(12, 64, 8, 2, 128), (12, 128, 32, 8, 128), (6, 256, 8, 2, 64), (12, 40, 4, 2, 128)])
+def test_block_prefill_layers_read_what_the_commit_wrote(monkeypatch, L, T, Hq, Hkv, D):
+    """Replays on changing projections (so that a stale cache would show) give what the same
+    launches give with a synchronisation after each, bit for bit: layers after the first start
+    early, but not before the commit two launches back is done."""
+    rng = np.random.default_rng(L * 1000 + T)
+    inputs = [[_bf16(rng, (L, 1, T, h, D)) for h in (Hq, Hkv, Hkv)] for _ in range(3)]
+    pf = BlockPrefill(L, 1, T, Hq, Hkv, D)
+    pf.load(*inputs[-1])
+    pf.step()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pf.step()
+    got = []
+    for x in inputs:
+        pf.load(*x)
+        graph.replay()
+        got.append([t.clone() for t in (pf.outp, pf.k_pages, pf.v_pages)])
+    torch.cuda.synchronize()
+    _synchronised(monkeypatch, "accept_commit")
+    _synchronised(monkeypatch, "verify_attn")
+    ref = BlockPrefill(L, 1, T, Hq, Hkv, D)
+    for x, have in zip(inputs, got):
+        ref.load(*x)
+        ref.step()
+        for a, b in zip(have, (ref.outp, ref.k_pages, ref.v_pages)):
+            assert torch.equal(a, b)
+    assert C.get_device_error() == 0
