@@ -366,9 +366,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         set_err(p.err, ERR_TIMEOUT);
         *abort_flag = 1;
       }
-      // every MMA issued by this warp's thread completes before TMEM is released
+      // (both CTAs wait for it below)
       umma_commit_pair_on(on, mma_done, 3);
-      mbar_wait(mma_done, 0, WAIT_NS);
     }
   } else {
     // ------------------------------------------------------------ epilogue
@@ -511,7 +510,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   tc_fence_before();
   __syncthreads();
   // Neither CTA leaves (or frees its TMEM) while the other may still signal its barriers or the
-  // pair's MMAs may write its TMEM.
+  // pair's MMAs may write its TMEM: the last signal of the leader's MMAs has arrived in both, and
+  // the barrier says so to each.
+  if (warp == 1) mbar_wait(mma_done, 0, WAIT_NS);
+  __syncwarp();
   cluster_arrive();
   cluster_wait();
   tc_fence_after();
