@@ -386,6 +386,11 @@ COSPEC_API int cospec_accept_commit(int B, int K, int num_layers, const cospec_a
                                     int32_t* ctx_len, int32_t* accept_len, int32_t* emitted,
                                     void* stream);
 
+/* Kernels such a call launches on the current device (0 for an empty batch): 1 where
+ * a sequence's layers are a cluster that also advances the context, else 2.
+ * Host only; a negative cospec_status for dimensions the call would refuse. */
+COSPEC_API int cospec_accept_commit_launches(const cospec_attn_dims* dims, int num_layers);
+
 /* ------------------------------------------------------------------------ */
 /* 5. RL stage: reward shaping, returns and advantages (Sec. 3.4).
  *

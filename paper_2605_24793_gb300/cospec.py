@@ -25,7 +25,7 @@ EXPORTED = ("cospec_status_string", "cospec_last_cuda_error", "cospec_get_device
             "cospec_arbitrate", "cospec_accept_commit", "cospec_lmhead_argmax_features_noalloc",
             "cospec_lmhead_sample_features", "cospec_verify_attn_plan", "cospec_rl_workspace",
             "cospec_rl_advantages", "cospec_verify_attn_plan_model",
-            "cospec_lmhead_logits_features", "cospec_sps_workspace", "cospec_sps_accept")
+            "cospec_lmhead_logits_features", "cospec_sps_workspace", "cospec_sps_accept", "cospec_accept_commit_launches")
 
 
 class AttnDims(ctypes.Structure):
@@ -96,6 +96,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         "cospec_arbitrate": (_i, [_i, _i, _vp, _vp, _vp, _i, _vp, _vp, _vp, _f, _f, _i, _vp, _vp, _vp]),
         "cospec_accept_commit": (_i, [_i, _i, _i, _PDIMS, _vp, _vp, _vp, _vp, _vp, _vp, _vp,
                                       ctypes.c_longlong, _vp, _vp, _vp, _vp, _vp]),
+        "cospec_accept_commit_launches": (_i, [_PDIMS, _i]),
     }
     for name, (res, args) in sig.items():
         fn = getattr(lib, name)
@@ -463,6 +464,14 @@ def arbitrate(draft, argmax, stats, w1, b1, w2, b2: float, lam: float, mode: int
         _ptr(b1) if mode == 0 else None, _ptr(w2) if mode == 0 else None, float(b2), float(lam),
         int(mode), _ptr(p_out), _ptr(accept), _stream(stream)))
     return p_out, accept
+
+
+def accept_commit_launches(dims: AttnDims, num_layers: int) -> int:
+    """Kernels accept_commit launches for a block of these dimensions."""
+    n = load_library().cospec_accept_commit_launches(ctypes.byref(dims), int(num_layers))
+    if n < 0:
+        _check(n)
+    return n
 
 
 def accept_commit(draft, argmax, accept, k_blk, v_blk, k_pages, v_pages, page_table, ctx_len,

@@ -484,4 +484,12 @@ COSPEC_API int cospec_accept_commit(int B, int K, int num_layers, const cospec_a
   return cuda_status(launch_accept_commit(a, err, static_cast<cudaStream_t>(stream)));
 }
 
+COSPEC_API int cospec_accept_commit_launches(const cospec_attn_dims* dims, int num_layers) {
+  const int st = check_attn_dims(dims);
+  if (st != COSPEC_OK) return st;
+  if (num_layers < 0) return COSPEC_ERR_INVALID_ARG;
+  if (dims->rows > 32) return COSPEC_ERR_UNSUPPORTED;
+  return accept_commit_launches(dims->batch, dims->rows - 1, num_layers, dims->num_kv_heads, dims->head_dim);
+}
+
 }  // extern "C"

@@ -168,5 +168,6 @@ struct CommitArgs {
   int32_t* emitted;
 };
 cudaError_t launch_accept_commit(const CommitArgs& a, int* err, cudaStream_t stream);
+int accept_commit_launches(int B, int K, int L, int Hkv, int D);   // kernels such a call launches
 
 }  // namespace cospec

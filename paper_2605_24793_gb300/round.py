@@ -111,11 +111,11 @@ class VerifyRound:
     def _count_launches(self) -> int:
         """Kernels one round launches (attention: 1 per layer; LM head: a main
         and a merge kernel per launch of up to four 256-row slices;
-        arbitration: 1 when K > 0; accept/commit: 1)."""
+        arbitration: 1 when K > 0; accept/commit: 1 or 2)."""
         cfg = self.cfg
         passes = (cfg.m_rows + 1023) // 1024
         decide = 2 if self.sps else (1 if cfg.k > 0 else 0)
-        return cfg.layers + 2 * passes + decide + 1
+        return cfg.layers + 2 * passes + decide + C.accept_commit_launches(self.dims, cfg.layers)
 
     def restore_context(self) -> None:
         """Reset ctx_len to the round's starting context (device copy)."""

@@ -703,6 +703,55 @@ def test_tcgen05_attention_device_checks_skip_only_the_bad_sequence():
     assert torch.all(out[1] == 0)                          # the skipped sequence attends nothing
 
 
+# Both sides of the rule for one launch or two: clusters of 1, 3, 8 and 8 (of two layers each) CTAs, the same
+# with too many CTAs or layers.
+@pytest.mark.parametrize("B,L,K,Hkv,launches", [
+    (3, 1, 4, 2, 1), (5, 3, 31, 8, 1), (4, 8, 7, 2, 1), (8, 16, 3, 2, 1), (2, 11, 0, 2, 1),
+    (9, 9, 3, 2, 2), (2, 17, 7, 2, 2), (110, 3, 2, 2, 2)])
+def test_accept_commit_launches_one_kernel_or_two(B, L, K, Hkv, launches):
+    rng = np.random.default_rng(B * 100 + L)
+    D, P, R, V = 64, 16, K + 1, 9
+    pages = 3
+    num = B * pages
+    table = rng.permutation(num).astype(np.int32).reshape(B, pages)
+    ctx = rng.integers(0, pages * P - R + 1, B).astype(np.int32)
+    am = rng.integers(0, V, (B, R)).astype(np.int32)
+    draft = np.where(rng.random((B, K)) < 0.6, am[:, :K], rng.integers(0, V, (B, K))).astype(np.int32)
+    acc = rng.integers(0, 2, (B, K)).astype(np.uint8)
+    kb, vb = bf16(rng.standard_normal((L, B, R, Hkv, D))), bf16(rng.standard_normal((L, B, R, Hkv, D)))
+    kp, vp = bf16(rng.standard_normal((L, num, Hkv, P, D))), bf16(rng.standard_normal((L, num, Hkv, P, D)))
+    bits = lambda x: x.cpu().view(torch.int16).numpy()
+    kp0, vp0 = bits(kp), bits(vp)
+    dims = C.AttnDims(B, R, Hkv, Hkv, D, P, pages, num, 0.0, 0)
+    assert C.accept_commit_launches(dims, L) == launches
+    ctx_t, alen = torch.from_numpy(ctx).cuda(), torch.empty(B, dtype=torch.int32, device="cuda")
+    am_t = torch.from_numpy(am).cuda()
+    # the emitted tokens may take the place of the target's
+    C.accept_commit(torch.from_numpy(draft).cuda(), am_t, torch.from_numpy(acc).cuda(), kb, vb, kp, vp,
+                    torch.from_numpy(table).cuda(), ctx_t, alen, am_t)
+    s, emitted = O.accept_scan(draft, am, acc)
+    kp_ref, vp_ref, ctx_ref = O.commit_kv(bits(kb), bits(vb), kp0, vp0, table, ctx, s, P)
+    assert np.array_equal(alen.cpu().numpy(), s) and np.array_equal(am_t.cpu().numpy(), emitted)
+    assert np.array_equal(ctx_t.cpu().numpy(), ctx_ref)
+    assert np.array_equal(bits(kp), kp_ref) and np.array_equal(bits(vp), vp_ref)
+    assert C.get_device_error() == 0
+
+
+def test_accept_commit_without_layers_takes_any_batch():
+    B, K = 70000, 3
+    z = lambda *sh: torch.zeros(sh, dtype=torch.int32, device="cuda")
+    kv, pool = (torch.zeros(sh, dtype=torch.bfloat16, device="cuda") for sh in ((0, B, K + 1, 2, 64), (1, 1, 2, 16, 64)))
+    ctx, alen, em = z(B), z(B), z(B, K + 1)
+    accept = torch.ones((B, K), dtype=torch.uint8, device="cuda")
+    accept[B - 1, 1] = 0
+    draft = z(B, K)
+    draft[B - 1, 1] = 5
+    C.accept_commit(draft, z(B, K + 1), accept, kv, kv.clone(), pool, pool.clone(), z(B, 1), ctx, alen, em)
+    assert C.get_device_error() == 0
+    assert (ctx[:-1] == K + 1).all() and int(ctx[-1]) == 2 and torch.equal(ctx, alen)
+    assert em[-1].tolist() == [0, 0, -1, -1]
+
+
 def test_accept_commit_device_checks_skip_only_the_bad_sequence():
     # Sequence 1 would run past its page table (ctx + s > capacity): its
     # context stays, nothing of it is written.  Sequence 2's commit page is
