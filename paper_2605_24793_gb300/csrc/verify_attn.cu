@@ -678,7 +678,7 @@ int variant_mt(int NR) {   // NR <= 64
 // rows per KV head, groups of 128 (one MMA row tile per CTA, 1 to 16 splits) or of 256, unsplit (two
 // row tiles sharing a K/V stream in one CTA, or a persistent CTA pair for head dimension 128), by the
 // smallest estimated time.  The estimates are as measured on GB300 (us): a CTA 7 + 0.94 per 128-key
-// tile, 3.5 more when split; two row tiles 7.5 + 1.9 per tile, whole waves of either at 15 % more from
+// tile, 4 more when split; two row tiles 7.5 + 1.9 per tile, whole waves of either at 15 % more from
 // the second on; a pair 3 and 4.4 + 0.79 per tile for each of its units.  They are put together for
 // equal contexts (whole waves, whole rounds of units) and for contexts that average 0.65 of the
 // longest (the longest CTA or unit, or the work spread over the resident clusters), weighted 0.35 to
@@ -713,7 +713,7 @@ static AttnPlan plan_tcq(const AttnPlan& base, int B, int R, int Hkv, int D, int
         longest = 3.0 + (4.4 + 0.79 * tiles);
         spread = 3.0 + (double)pl.units / fit * (4.4 + 0.79 * 0.65 * tiles);
       } else {
-        const double per_tile = two ? 1.9 : 0.94, start = two ? 7.5 : s > 1 ? 10.5 : 7.0;
+        const double per_tile = two ? 1.9 : 0.94, start = two ? 7.5 : s > 1 ? 11.0 : 7.0;
         longest = start + per_tile * ((tiles + s - 1) / s);
         equal = waves * longest * (waves > 1 ? 1.15 : 1.0);
         spread = (double)pl.units / fit * (start + per_tile * 0.65 * tiles / s);

@@ -30,7 +30,7 @@
 // relative to m_ref, set exactly by the first tile; a later tile moves m_ref (and
 // rescales O_h and l) only when one of its scores exceeds it by more than
 // 2^8 in the exp2 domain, so P stays below 256 and rescales are rare.
-// With SWAP (clusters of eight or more CTAs: a few tiles each) the two threads of a row swap
+// With SWAP (D = 128, split, up to three tiles per CTA) the two threads of a row swap
 // their half maxima through shared memory every tile instead and share one reference,
 // sum and accumulator O, with a third score buffer in the room that is left; nothing is
 // left to put together at the end.
@@ -868,19 +868,28 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
       const int j = j0 + (rvalid ? r / p.G : 0), g = rvalid ? r % p.G : 0;
       __nv_bfloat16* dst = p.out + (((size_t)b * p.R + j) * p.Hq + (size_t)kvh * p.G + g) * D;
       const float inv = (have && l > 0.f) ? 1.f / l : 0.f;
+      // (16 columns at a time, not unrolled: this code runs once, and its fetch showed, 7.6 -> 7.1 us
+      // at batch 1 and 100 keys)
+#pragma unroll 1
+      for (int c = 2 * c0; c < 2 * c0 + D / 32; ++c) {
+        float o[16], o1[16];
+        if (have) {
+          tq_ld16(orow + c * 16, o);
+          if (have1) tq_ld16(orow + D + c * 16, o1);
+          tq_wait_ld();
+        }
 #pragma unroll
-      for (int c = c0; c < c0 + D / 64; ++c) {
-        float o[32];
-        load_o(c, o);
+        for (int i = 0; i < 16; ++i)
+          o[i] = !have ? 0.f : SWAP ? o[i] : have1 ? o[i] * w0_ + o1[i] * w1_ : o[i] * w0_;
         if (rvalid) {
 #pragma unroll
-          for (int i = 0; i < 32; i += 8) {
+          for (int i = 0; i < 16; i += 8) {
             uint4 w;
             w.x = pack_bf16(o[i] * inv, o[i + 1] * inv);
             w.y = pack_bf16(o[i + 2] * inv, o[i + 3] * inv);
             w.z = pack_bf16(o[i + 4] * inv, o[i + 5] * inv);
             w.w = pack_bf16(o[i + 6] * inv, o[i + 7] * inv);
-            *reinterpret_cast<uint4*>(dst + c * 32 + i) = w;
+            *reinterpret_cast<uint4*>(dst + c * 16 + i) = w;
           }
         }
       }
@@ -1105,17 +1114,15 @@ cudaError_t launch_verify_attn_tcq(const AttnArgs& a, const AttnPlan& pl, int* e
   p.kv_stable = a.kv_stable;
   p.block_full = a.block_full;
   p.err = err;
-  // Eight or more CTAs per cluster (batch 1) have two or three tiles each, where the halves' own
-  // accumulators cost more at the end than the swaps on the way: 10.05 us per layer against 9.79
-  // (K = 15) and 11.2 against 10.85 (K = 25); from batch 2 on (longer runs of tiles) they gain, 12.40
-  // against 12.47 and, at batch 4, 18.9 against 19.2.
-  const bool swap = pl.cluster >= 8;
+  // Split with up to three tiles per CTA, the halves' own accumulators cost more at the end than
+  // the swaps on the way.  Swapping against halves, time per layer back to back at D = 128, batches 1 to
+  // 64, 100 to 8192 keys, by tiles per CTA: 1 0.97-0.99, 2 0.96-1.01, 3 0.97-0.98, 4 0.98-1.03, more
+  // 1.00-1.04; unsplit 1.01-1.06; at D = 64, whose products are half as long, 1.01-1.24 throughout.
+  const int tiles = (a.max_ctx + QKT - 1) / QKT, S = pl.cluster;
   if (a.D == 128)
-    return swap ? launch_tcq_t<128, true>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream)
-                : launch_tcq_t<128, false>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream);
-  if (a.D == 64)
-    return swap ? launch_tcq_t<64, true>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream)
-                : launch_tcq_t<64, false>(maps, p, pl.cluster, a.B, a.Hkv, pl.rg, stream);
+    return S > 1 && (tiles + S - 1) / S <= 3 ? launch_tcq_t<128, true>(maps, p, S, a.B, a.Hkv, pl.rg, stream)
+                                             : launch_tcq_t<128, false>(maps, p, S, a.B, a.Hkv, pl.rg, stream);
+  if (a.D == 64) return launch_tcq_t<64, false>(maps, p, S, a.B, a.Hkv, pl.rg, stream);
   return cudaErrorInvalidValue;
 }
 

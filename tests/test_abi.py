@@ -121,6 +121,8 @@ PLAN_CASES = [
     ((16, 16, 32, 8, 128, 8192, 1), (C.ATTN_TCGEN05, 2)),   # batch 16, K = 15
     ((32, 8, 64, 8, 128, 16384, 1), (C.ATTN_TCGEN05, 1)),   # Qwen3-32B, batch 32
     ((64, 8, 32, 8, 128, 32768, 1), (C.ATTN_MMA_SYNC, 2)),  # Llama-3-8B, batch 64
+    ((8, 26, 32, 8, 128, 1024, 1), (C.ATTN_TCGEN05, 1)),    # 64 units of 8 tiles: unsplit 15.3 us, 2 splits 16.8
+    ((32, 64, 4, 2, 128, 1024, 1), (C.ATTN_TCGEN05, 1)),    # the same with 128 rows: 15.9 against 17.8
 ]
 
 
