@@ -91,29 +91,22 @@ class BlockPrefill:
         step = self.rows // chunk
         self.block_table = self.table2[::step].contiguous()
         self.block_start = self.start[::step].contiguous()
-        # chunk-padded projections [L, B, nck * chunk, H, D]; whole chunks need them for inputs
-        # that cannot be read in place only, and have no padding rows to be zero
-        self.qp = self.kp = self.vp = self.outp = None
-        if context != self.nck * chunk:
-            self._padded()
+        # chunk-padded projections [L, B, nck * chunk, H, D]: made here, so that a step
+        # captured into a graph reads what later loads place in them
+        padded = lambda heads: torch.zeros((layers, batch, self.nck * chunk, heads, head_dim),
+                                           dtype=torch.bfloat16, device=dev)
+        self.qp, self.kp, self.vp = padded(q_heads), padded(kv_heads), padded(kv_heads)
+        self.outp = torch.empty_like(self.qp)
 
     def _check(self, q, k, v) -> None:
         L, B, C = self.L, self.B, self.C
         if tuple(q.shape) != (L, B, C, self.Hq, self.D) or tuple(k.shape) != (L, B, C, self.Hkv, self.D):
             raise ValueError("q / k / v must be [L, B, C, H, D] with the prefill's shape")
 
-    def _padded(self) -> None:
-        if self.qp is None:
-            padded = lambda heads: torch.zeros((self.L, self.B, self.nck * self.chunk, heads, self.D),
-                                               dtype=torch.bfloat16, device=self.k_pages.device)
-            self.qp, self.kp, self.vp = padded(self.Hq), padded(self.Hkv), padded(self.Hkv)
-            self.outp = torch.empty_like(self.qp)
-
     def load(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> None:
         """q [L, B, C, Hq, D], k / v [L, B, C, Hkv, D] (bf16): the context's
         per-layer projections, placed into the chunk-padded buffers."""
         self._check(q, k, v)
-        self._padded()
         # v may have more rows than the context, or broadcast: then chunk by chunk
         n = max(1, self.C) if v.shape == k.shape else self.chunk
         for dst, src in ((self.qp, q), (self.kp, k), (self.vp, v)):
@@ -124,7 +117,6 @@ class BlockPrefill:
     def step(self) -> None:
         """The prefill itself, from the loaded buffers: one commit, then one
         attention launch per layer (all launches, no host synchronisation)."""
-        self._padded()
         self._launch(self.qp, self.kp, self.vp, self.outp)
 
     def _launch(self, q, k, v, out) -> None:

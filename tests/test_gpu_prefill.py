@@ -150,3 +150,23 @@ def test_block_prefill_layers_read_what_the_commit_wrote(monkeypatch, L, T, Hq, 
         for a, b in zip(have, (ref.outp, ref.k_pages, ref.v_pages)):
             assert torch.equal(a, b)
     assert C.get_device_error() == 0
+
+
+@pytest.mark.parametrize("T", [64, 72])
+def test_block_prefill_step_captured_before_any_load(T):
+    """A step captured first, projections loaded afterwards: each replay takes those."""
+    L, Hq, Hkv, D = 2, 4, 2, 64
+    rng = np.random.default_rng(T)
+    pf, ref = BlockPrefill(L, 1, T, Hq, Hkv, D), BlockPrefill(L, 1, T, Hq, Hkv, D)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pf.step()
+    for _ in range(2):
+        x = [_bf16(rng, (L, 1, T, h, D)) for h in (Hq, Hkv, Hkv)]
+        pf.load(*x)
+        graph.replay()
+        out = ref.run(*x)
+        torch.cuda.synchronize()
+        assert torch.equal(pf.outp[:, :, :T], out)
+        assert torch.equal(pf.k_pages, ref.k_pages) and torch.equal(pf.v_pages, ref.v_pages)
+    assert C.get_device_error() == 0
