@@ -15,9 +15,9 @@ target's, so the accepted length is the chunk's length).
   "sequences" are the chunks (each with its sequence's page-table row and its
   start as context length), and then attends all chunks of a layer in one
   verify-attention launch: chunk k sees exactly the positions before it.  The
-  chunks lie in the context's own order, so a context of whole chunks needs no
-  copy (placing chunk by chunk took 512 copy launches and 7.9 ms of the 8.5 ms
-  of a 4-layer, 4096-token call).
+  chunks lie in the context's own order, so that one copy per tensor places them
+  (chunk by chunk it took 512 copy launches and 7.9 ms of the 8.5 ms of a
+  4-layer, 4096-token call) and a context of whole chunks needs none for its output.
 * ``ChunkedPrefill`` walks the chunks one after another (attention of every
   layer, then the commit), the plain reference for the block driver.
 
@@ -138,17 +138,14 @@ class BlockPrefill:
 
     def run(self, q: torch.Tensor, k: torch.Tensor, v: torch.Tensor) -> torch.Tensor:
         """Commits the context's K/V into the cache and returns the attention
-        output [L, B, C, Hq, D].  A context of whole chunks is read and written
-        where it lies; a ragged one, and projections of another device, type or
-        layout, go through the padded buffers."""
-        self._check(q, k, v)
+        output [L, B, C, Hq, D].  The projections stay loaded for a later step();
+        the output of a context of whole chunks is written where it is returned."""
+        self.load(q, k, v)
         out = torch.empty_like(q)
-        if self.C == self.nck * self.chunk and v.shape == k.shape and all(
-                t.device == self.k_pages.device and t.is_contiguous() and t.dtype == torch.bfloat16
-                and t.data_ptr() % 16 == 0 for t in (q, k, v)):
-            self._launch(q, k, v, out)
+        if (self.C == self.nck * self.chunk and out.device == self.k_pages.device and out.is_contiguous()
+                and out.dtype == torch.bfloat16):
+            self._launch(self.qp, self.kp, self.vp, out)
         else:
-            self.load(q, k, v)
             self.step()
             out.copy_(self.outp[:, :, :self.C])
         return out

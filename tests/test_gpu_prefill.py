@@ -170,3 +170,21 @@ def test_block_prefill_step_captured_before_any_load(T):
         assert torch.equal(pf.outp[:, :, :T], out)
         assert torch.equal(pf.k_pages, ref.k_pages) and torch.equal(pf.v_pages, ref.v_pages)
     assert C.get_device_error() == 0
+
+
+@pytest.mark.parametrize("T", [64, 72])
+def test_block_prefill_run_leaves_its_projections_loaded(T):
+    """A step() after run() is the same prefill again, whatever became of the inputs."""
+    L, Hq, Hkv, D = 2, 4, 2, 64
+    rng = np.random.default_rng(T + 1)
+    pf = BlockPrefill(L, 1, T, Hq, Hkv, D)
+    x = [_bf16(rng, (L, 1, T, h, D)) for h in (Hq, Hkv, Hkv)]
+    out = pf.run(*x)
+    kp, vp = pf.k_pages.clone(), pf.v_pages.clone()
+    for t in x:
+        t.zero_()
+    pf.step()
+    torch.cuda.synchronize()
+    assert torch.equal(pf.outp[:, :, :T], out)
+    assert torch.equal(pf.k_pages, kp) and torch.equal(pf.v_pages, vp)
+    assert C.get_device_error() == 0
