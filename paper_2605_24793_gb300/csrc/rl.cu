@@ -129,7 +129,7 @@ CS_DEV F2 warp_sum(F2 v) {
 }
 
 // log of a normal positive float as a pair, by table (Tang, ACM TOMS 1990): x = 2^e m with m in
-// [0.707, 1.414), inv ~ 1 / m a multiple of 2^-8 (so that r = m inv - 1 is exact, |r| <= 2^-7),
+// [0.707, 1.414), inv ~ 1 / m a multiple of 2^-8, r = m inv - 1 with |r| <= 2^-7 (25 bits: a pair),
 //   log x = e log 2 - log inv + log(1 + r),   log(1 + r) = r - r^2/2 + r^3 (1/3 - r/4 + ...).
 // Around m = 1 inv is 1, so log(1 + r) keeps its relative accuracy there.
 // Entry j - 90 (j = floor(128 m)): inv, -log inv in two parts.
@@ -208,7 +208,8 @@ CS_DEV F2 log_pair(float x, const float (*tab)[3]) {
     ++e;
   }
   const float* t = tab[(int)(m * 128.f) - 90];
-  const F2 lr = log1p_small(F2{fmaf(m, t[0], -1.f), 0.f});
+  const F2 mi = two_prod(m, t[0]);
+  const F2 lr = log1p_small(two_sum(__fsub_rn(mi.h, 1.f), mi.l));
   // log 2 in three parts, the first of 16 bits (e times it is exact)
   const float fe = (float)e;
   const F2 b = two_prod(fe, 0x1.7f7d1cp-20f);

@@ -157,6 +157,31 @@ def test_sums_keep_their_precision(K, policy):
     assert C.get_device_error() == 0
 
 
+@pytest.mark.parametrize("K", [1, 3])
+def test_entropy_and_kl_of_single_decisions(K):
+    """One decision a call, so that nothing averages out: the result's 32-bit rounding (2^-24) and the
+    pairs' error (logarithms to 3e-14, against an entropy of at least 0.03 and a KL of at least 5e-6
+    here: 1e-8) are all that may show.  The relative steps from p to q lie where the KL changes from
+    log(1 + r) to the difference of two logarithms (r = 2^-6) and well to both sides."""
+    rng = np.random.default_rng(K)
+    n = 200
+    p = rng.uniform(0.05, 0.95, n).astype(np.float32)
+    q = (p * (1 + rng.choice([-1, 1], n) * rng.uniform(0.01, 0.05, n))).astype(np.float32)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")
+    match, one = torch.zeros((1, K), dtype=torch.uint8, device="cuda"), torch.ones((1, K), device="cuda")
+    accept = torch.zeros((1, K), dtype=torch.uint8, device="cuda")       # the first position is rejected: one decision
+    ld = np.longdouble
+    for a, b in zip(p, q):
+        out = C.rl_advantages(i32([0, 1]), torch.ones(1, dtype=torch.uint8, device="cuda"), i32([0, 1]), match, accept, one,
+                              None, one, torch.full((1, K), float(a), device="cuda"), torch.full((1, K), float(b), device="cuda"))
+        loss = out["loss"].double().cpu().numpy()
+        P, Q = ld(a), ld(b)
+        ent = -P * np.log(P) - (1 - P) * np.log1p(-P)
+        kl = P * np.log1p((P - Q) / Q) + (1 - P) * np.log1p((Q - P) / (1 - Q))
+        assert abs(loss[1] - ent) <= (2.0 ** -24 + 1e-8) * ent
+        assert abs(loss[2] - kl) <= (2.0 ** -24 + 1e-8) * kl
+
+
 def test_infinities_and_nan_pass_through():
     rng = np.random.default_rng(3)
     batch = _sized_batch(rng, 25)
