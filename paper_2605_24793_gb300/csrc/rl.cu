@@ -12,8 +12,10 @@
 //    every large access is a run of consecutive addresses;
 //  - per-position values stay in 32 bits where that is exact (g, rho) and in
 //    pairs of 32-bit floats (about 2^-46 relative) where the result needs more:
-//    the sums of |g|, the decision advantages, and the logarithms, products and
-//    sums of the entropy and the KL divergence;
+//    the decision advantages, and the logarithms, products and sums of the entropy
+//    and the KL divergence; a round's share of the return and the sums of these are
+//    in 64 bits (a few operations per round: returns that differ in their last bits alone
+//    decide a standardisation whose sigma is as small);
 //  - the effective decisions (a fifth of all positions) are compacted through
 //    a per-warp queue, so that the objective's arithmetic runs on full warps;
 //  - inputs outside the range where the pairs hold (infinities, NaN, huge or
@@ -357,7 +359,9 @@ __global__ void __launch_bounds__(RL_THREADS, 2) rl_group_kernel(const RLArgs a)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int K = a.K;
   __shared__ unsigned long long s_eff[RL_TILE], s_acc[RL_TILE];
-  __shared__ F2 s_val[RL_TILE];          // a round's share of the return; its decisions' factor
+  __shared__ double s_ret[RL_TILE];      // a round's share of the return
+  __shared__ F2 s_val[RL_TILE];          // its decisions' factor
+  __shared__ double s_rcp[65];           // 1 / i
   __shared__ float s_rho[RL_TILE];
   __shared__ uint8_t s_stop[RL_TILE];    // s, with bit 7: the rollout is correct
   __shared__ uint8_t s_big[RL_TILE];     // the round's return takes the general path
@@ -386,6 +390,7 @@ __global__ void __launch_bounds__(RL_THREADS, 2) rl_group_kernel(const RLArgs a)
     a.ws_j[m] = 0.0;
     a.ws_abs[m] = 0.0;
   }
+  for (int i = 1 + tid; i <= K; i += RL_THREADS) s_rcp[i] = 1.0 / (double)i;
   if (a.part)
     for (int i = tid; i < 91 * 3; i += RL_THREADS) (&s_tab[0][0])[i] = (&RL_LOG_TAB[0][0])[i];
   some_bad = __syncthreads_or(some_bad) != 0;
@@ -428,23 +433,30 @@ __global__ void __launch_bounds__(RL_THREADS, 2) rl_group_kernel(const RLArgs a)
         // num / den of small whole numbers: the 32-bit quotient is the 64-bit one rounded
         const float rho = k.istar ? __fdiv_rn((float)num, (float)den) : 0.f;
         a.rho[r] = k.istar ? rho : __int_as_float(0x7fc00000);
-        F2 v{0.f, 0.f};
+        // this round's share of the return, to 64 bits: n rho from a table of reciprocals, or the
+        // accepted |ell| in three floats (each two-sum's rounding goes into the next)
+        double v = 0.0;
         bool big = false;
-        if (corr) {                      // n rho
-          if (k.istar) v = div(F2{(float)(k.n * num), 0.f}, F2{(float)den, 0.f});
-        } else {                         // the accepted |ell|
+        if (corr) {
+          if (k.istar) v = (double)(k.n * num) * s_rcp[den];
+        } else {
+          float v0 = 0.f, v1 = 0.f, v2 = 0.f;
           for (unsigned long long left = k.eff; left; left &= left - 1) {
             const int i = __ffsll((long long)left) - 1;
             const float l = fabsf(a.ell[e0 + i]);
             big |= !(alpha_ok && l < 1e20f);
-            const F2 t = two_sum(v.h, ((k.acc >> i) & 1) ? l : 0.f);
-            v = quick_two_sum(t.h, __fadd_rn(v.l, t.l));
+            const F2 t = two_sum(v0, ((k.acc >> i) & 1) ? l : 0.f);
+            const F2 u = two_sum(v1, t.l);
+            v0 = t.h;
+            v1 = u.h;
+            v2 += u.l;
           }
+          v = (double)v0 + ((double)v1 + (double)v2);
         }
         s_eff[tid] = k.eff;
         s_acc[tid] = k.acc;
         s_rho[tid] = rho;
-        s_val[tid] = v;
+        s_ret[tid] = v;
         s_stop[tid] = (uint8_t)(k.s | (corr ? 128 : 0));
         s_big[tid] = big;
       }
@@ -479,14 +491,14 @@ __global__ void __launch_bounds__(RL_THREADS, 2) rl_group_kernel(const RLArgs a)
       for (int m = mf + warp; m <= ml; m += RL_WARPS) {
         const int b0 = max(a.round_off[m], t0) - t0, b1 = min(a.round_off[m + 1], t0 + nr) - t0;
         const bool corr = a.correct[m] != 0;
-        F2 v{0.f, 0.f};
+        double v = 0.0;
         int rejected = 0;
         bool wide = false;
         double dg = 0.0, da = 0.0;
         for (int r = b0 + lane; r < b1; r += 32) {
           const int stop = s_stop[r] & 127;
           if (!s_big[r]) {
-            v = add(v, s_val[r]);
+            v += s_ret[r];
             rejected += stop <= K ? 1 : 0;
             continue;
           }
@@ -506,7 +518,7 @@ __global__ void __launch_bounds__(RL_THREADS, 2) rl_group_kernel(const RLArgs a)
           da = warp_sum(da);
         }
         if (lane == 0) {
-          const double s = to_double(v), rj = (double)rejected;
+          const double s = v, rj = (double)rejected;
           a.ws_j[m] += corr ? s : dg - (alpha * s + beta * rj);
           a.ws_abs[m] += corr ? s : da + (fabs(alpha) * s + fabs(beta) * rj);
         }
