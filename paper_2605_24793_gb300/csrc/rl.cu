@@ -2,11 +2,11 @@
 // returns, rebalanced group-normalised advantages, per-decision advantages
 // and the clipped objective with its entropy and KL terms.
 //
-// One CTA of 16 warps per prompt group.  The call is bound by memory (27
+// One CTA of 16 warps (4 for many small groups) per prompt group.  The call is bound by memory (27
 // bytes per decision with the objective) as long as two things stay off its
 // path: uncoalesced access and 64-bit arithmetic, of which an SM issues only
 // about two multiply-adds per clock.  So
-//  - a CTA works on tiles of 512 rounds.  A thread takes one round to find s,
+//  - a CTA works on tiles of a round per thread.  A thread takes its round to find s,
 //    i* and the effective set (its K flags become bit masks, four flags per
 //    instruction), and the tile's decisions are then walked in memory order, so
 //    every large access is a run of consecutive addresses;
@@ -29,7 +29,7 @@
 // Measured (GB300, 256 prompts x 8 rollouts of up to 64 rounds at K = 25, 1.66 M
 // decisions with the objective; time of the call's kernels): a lane per round
 // walking its K bytes, everything in 64 bits, 790 us; a warp per round with
-// ballots and pairs 95-107 us; this split 48.7 us (0.9 TB/s, instruction-bound:
+// ballots and pairs 95-107 us; this split 49.5 us (0.9 TB/s, instruction-bound:
 // about 330 warp instructions a round).  The call's host side takes 47 us.
 #include <math.h>
 
@@ -41,9 +41,6 @@ namespace cospec {
 
 namespace {
 
-constexpr int RL_THREADS = 512;
-constexpr int RL_WARPS = RL_THREADS / 32;
-constexpr int RL_TILE = RL_THREADS;      // rounds per tile, one per thread
 constexpr int RL_LOSS_THREADS = 256;
 
 struct RLArgs {
@@ -220,6 +217,14 @@ CS_DEV F2 log_pair(float x, const float (*tab)[3]) {
   return add(s, lr);
 }
 
+struct RLReciprocals {
+  double v[65];
+  constexpr RLReciprocals() : v{} {
+    for (int i = 1; i <= 64; ++i) v[i] = 1.0 / i;
+  }
+};
+__device__ const RLReciprocals RL_RCP;   // 1 / i
+
 CS_DEV double bern_entropy(double p) {
   double h = 0.0;
   if (p > 0.0) h -= p * log(p);
@@ -354,14 +359,16 @@ CS_DEV int rollout_of(const int32_t* round_off, int ma, int mb, int r) {
   return lo;
 }
 
-__global__ void __launch_bounds__(RL_THREADS, 2) rl_group_kernel(const RLArgs a) {
+template <int RL_THREADS>
+__global__ void __launch_bounds__(RL_THREADS, 1024 / RL_THREADS) rl_group_kernel(const RLArgs a) {
+  constexpr int RL_WARPS = RL_THREADS / 32;
+  constexpr int RL_TILE = RL_THREADS;    // rounds per tile, one per thread
   const int x = blockIdx.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int K = a.K;
   __shared__ unsigned long long s_eff[RL_TILE], s_acc[RL_TILE];
   __shared__ double s_ret[RL_TILE];      // a round's share of the return
   __shared__ F2 s_val[RL_TILE];          // its decisions' factor
-  __shared__ double s_rcp[65];           // 1 / i
   __shared__ float s_rho[RL_TILE];
   __shared__ uint8_t s_stop[RL_TILE];    // s, with bit 7: the rollout is correct
   __shared__ uint8_t s_big[RL_TILE];     // the round's return takes the general path
@@ -390,7 +397,6 @@ __global__ void __launch_bounds__(RL_THREADS, 2) rl_group_kernel(const RLArgs a)
     a.ws_j[m] = 0.0;
     a.ws_abs[m] = 0.0;
   }
-  for (int i = 1 + tid; i <= K; i += RL_THREADS) s_rcp[i] = 1.0 / (double)i;
   if (a.part)
     for (int i = tid; i < 91 * 3; i += RL_THREADS) (&s_tab[0][0])[i] = (&RL_LOG_TAB[0][0])[i];
   some_bad = __syncthreads_or(some_bad) != 0;
@@ -438,7 +444,7 @@ __global__ void __launch_bounds__(RL_THREADS, 2) rl_group_kernel(const RLArgs a)
         double v = 0.0;
         bool big = false;
         if (corr) {
-          if (k.istar) v = (double)(k.n * num) * s_rcp[den];
+          if (k.istar) v = (double)(k.n * num) * RL_RCP.v[den];
         } else {
           float v0 = 0.f, v1 = 0.f, v2 = 0.f;
           for (unsigned long long left = k.eff; left; left &= left - 1) {
@@ -772,7 +778,14 @@ extern "C" COSPEC_API int cospec_rl_advantages(
   a.part = have_obj ? reinterpret_cast<double*>(base + 3 * mb) : nullptr;
   a.err = err;
   if (num_groups > 0) {
-    const cudaError_t e = launch_pdl(rl_group_kernel, dim3(num_groups), dim3(RL_THREADS), 0, st, a);
+    // Many small groups (more than a wave of 512-thread CTAs, at most 2048 decisions each) in CTAs of 128
+    // threads, eight to an SM: a CTA then waits on its own chain of loads and sums more than it
+    // works.  us, 512 -> 128 threads: 512 groups of 1.5 rounds, K = 3 24.3 -> 14.0; 2048 of 10, K = 5,
+    // with the objective 109 -> 49.5; 512 of 34, K = 31 49.5 -> 35.2.  Beyond: 512 of 132, K = 31
+    // (4092 decisions) 69 -> 84; 152 of 34, K = 25 24.3 -> 31.1.
+    const bool small = num_groups > 2 * device_num_sms() && (long long)num_rounds * K <= 2048LL * num_groups;
+    const cudaError_t e = small ? launch_pdl(rl_group_kernel<128>, dim3(num_groups), dim3(128), 0, st, a)
+                                : launch_pdl(rl_group_kernel<512>, dim3(num_groups), dim3(512), 0, st, a);
     if (e != cudaSuccess) return cuda_status(e);
   }
   if (have_obj) {

@@ -201,6 +201,24 @@ def test_equal_returns_in_another_order_stay_equal():
         assert np.abs(got["adv"]).max() <= 18 * 2.0 ** -53 * J / 1e-6
 
 
+@pytest.mark.parametrize("K,sizes,rounds", [
+    (3, (1, 0, 2), (0, 1, 2)), (5, (4,), (1, 2, 3, 4)), (64, (1, 2), (0, 1, 33)), (7, (5, 1), (33, 70)), (31, (2, 3), (20, 33))])
+def test_many_small_groups(K, sizes, rounds):
+    """Both sides of the rule for small CTAs (more than 304 groups of at most 2048 decisions on average),
+    groups of several tiles of 128 rounds among them."""
+    rng = np.random.default_rng(K)
+    batch = _sized_batch(rng, K, sizes=sizes * 160, rounds=rounds)
+    R = batch[4].shape[0]
+    ratio, p_new, p_ref = (rng.uniform(0.05, 0.95, (R, K)).astype(np.float32) for _ in range(3))
+    got = _run(batch, (ratio, p_new, p_ref))
+    ref = RL.rl_advantages(*batch, _f32_params(), ratio=ratio, p_new=p_new, p_ref=p_ref)
+    assert np.array_equal(got["eff"], ref["eff"])
+    for k in ("g", "rho", "J", "Jbar", "adv", "adv_dec"):
+        np.testing.assert_allclose(got[k], ref[k], rtol=1e-6, atol=1e-9 * np.nanmax(np.abs(ref[k])), err_msg=k)
+    np.testing.assert_allclose(got["loss"], np.array(ref["loss_terms"]), rtol=1e-6)
+    assert C.get_device_error() == 0
+
+
 def test_infinities_and_nan_pass_through():
     rng = np.random.default_rng(3)
     batch = _sized_batch(rng, 25)
