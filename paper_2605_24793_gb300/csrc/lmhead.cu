@@ -547,8 +547,12 @@ __global__ void __launch_bounds__(128) lmhead_reduce_kernel(const float4* part, 
   if (lane == 0) {
     const int m = row0 + row;
     float* st = stats + (size_t)m * 5;
+    if (a.m == INFINITY && a.sec < INFINITY && a.s == INFINITY) {   // one logit is infinite: all the weight
+      a.s = 1.f;
+      a.t = 0.f;
+    }
     const float ls = logf(a.s);
-    argmax[m] = a.i;
+    argmax[m] = a.i < V ? a.i : 0;         // no logit above -inf: the lowest id
     st[0] = a.m;
     st[1] = a.sec;
     st[2] = a.m + ls;

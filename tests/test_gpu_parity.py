@@ -797,6 +797,43 @@ def test_accept_commit_device_checks_skip_only_the_bad_sequence():
         assert np.array_equal(vp_got[:, pages], vp_ref[:, pages])
 
 
+@pytest.mark.parametrize("mode", ["greedy", "sampled", "logits"])
+@pytest.mark.parametrize("M,V", [(3, 300), (40, 257), (300, 1000)])
+def test_lmhead_infinite_and_nan_rows(mode, M, V):
+    """Rows whose logits are all -inf, or all NaN, still name an id of the vocabulary; one infinite
+    logit takes all the weight; the other rows are as without them."""
+    rng = np.random.default_rng(M + V)
+    d = 64
+    hidden = bf16(rng.standard_normal((M, d)))
+    w = bf16(rng.random((V, d)) + 0.5)
+    bad = hidden.clone()
+    w[17, 9] = -1.0
+    bad[0, 5], bad[M - 1, 7] = -math.inf, math.nan
+    bad[M // 2, 9] = -math.inf           # id 17: +inf, all others -inf
+
+    def run(h):
+        ids = torch.empty(M, dtype=torch.int32, device="cuda")
+        st = torch.empty((M, 5), dtype=torch.float32, device="cuda")
+        dfr, ws = torch.full((M,), -1, dtype=torch.int32, device="cuda"), C.new_lmhead_workspace(M, d, V)
+        if mode == "greedy":
+            C.lmhead_argmax_features(h, w, dfr, ids, st, ws)
+        elif mode == "sampled":
+            C.lmhead_sample_features(h, w, dfr, 1.0, torch.tensor([5], device="cuda"), ids, st, ws)
+        else:
+            C.lmhead_logits_features(h, w, dfr, 1.0, ids, st, torch.empty((M, V), device="cuda"), ws)
+        return ids.cpu().numpy(), st[:, :4].cpu().numpy()
+
+    ids, st = run(bad)
+    ref_ids, ref_st = run(hidden)
+    rows = [0, M // 2, M - 1]
+    assert ids[rows].tolist() == [0, 17, 0] and st[0, 0] == -math.inf and math.isnan(st[M - 1, 2])
+    assert st[M // 2].tolist() == [math.inf, -math.inf, math.inf, 0.0]
+    keep = np.setdiff1d(np.arange(M), rows)
+    assert np.array_equal(ids[keep], ref_ids[keep]) and np.array_equal(st[keep], ref_st[keep])
+    assert C.get_device_error() == 0
+
+
+
 # ---------------------------------------------------------------------------
 # Stochastic decoding: temperature sampling in the LM-head epilogue (Sec. 3.1)
 # ---------------------------------------------------------------------------
