@@ -391,6 +391,14 @@ CS_DEV void tq_wait_ld32(float (&v)[32]) {
                :
                : "memory");
 }
+CS_DEV void tq_wait_ld16(float (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]),
+                 "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]),
+                 "+f"(v[14]), "+f"(v[15])
+               :
+               : "memory");
+}
 CS_DEV void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   tq_ld32(taddr, v);
   tq_wait_ld32(v);

@@ -449,17 +449,36 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if ((unsigned)at < 32u && draft[c] < p.V)
           p.stats[(size_t)(row0 + ch * 32 + lane) * 5 + 4] = xp[xp_off(lane, at)];
         if (KEYED) {
-          tmem_ld32(tbase + (uint32_t)(ch * 32), x);
+          // 16 columns at a time, not unrolled: eight generators' code for each of four chunks was
+          // fetched more slowly than it ran (us, d 64, V 128: 8 rows 11.3 -> 8.6, 200 rows 35.2 -> 19.5; d 1024,
+          // V 32003: 256 rows 53.6 -> 40.0); columns past the last 16 with a row draw nothing
+          __syncwarp();
+#pragma unroll 1
+          for (int j0 = 0; j0 < 32 && ch * 32 + j0 < n_rows; j0 += 16) {
+            float k16[16];
+            tq_ld16(tbase + (uint32_t)(ch * 32 + j0), k16);
+            tq_wait_ld16(k16);
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) {
+              const uint4 u = philox4x32_10(
+                  make_uint4((uint32_t)(v0 + lane), (uint32_t)((row0 + ch * 32 + j0 + j) >> 2), 0u, 0u), seed_lo, seed_hi);
+              k16[j + 0] = fmaf(k16[j + 0], p.inv_temp, gumbel_of(u.x));
+              k16[j + 1] = fmaf(k16[j + 1], p.inv_temp, gumbel_of(u.y));
+              k16[j + 2] = fmaf(k16[j + 2], p.inv_temp, gumbel_of(u.z));
+              k16[j + 3] = fmaf(k16[j + 3], p.inv_temp, gumbel_of(u.w));
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) xp[xp_off(j0 + j, lane)] = valid ? k16[j] : -INFINITY;
+          }
+          __syncwarp();
 #pragma unroll
           for (int j = 0; j < 32; j += 4) {
-            const uint4 u = philox4x32_10(
-                make_uint4((uint32_t)(v0 + lane), (uint32_t)((row0 + ch * 32 + j) >> 2), 0u, 0u), seed_lo, seed_hi);
-            x[j + 0] = fmaf(x[j + 0], p.inv_temp, gumbel_of(u.x));
-            x[j + 1] = fmaf(x[j + 1], p.inv_temp, gumbel_of(u.y));
-            x[j + 2] = fmaf(x[j + 2], p.inv_temp, gumbel_of(u.z));
-            x[j + 3] = fmaf(x[j + 3], p.inv_temp, gumbel_of(u.w));
+            const float4 v = *reinterpret_cast<const float4*>(xp + xp_off(lane, j));
+            x[j] = v.x;
+            x[j + 1] = v.y;
+            x[j + 2] = v.z;
+            x[j + 3] = v.w;
           }
-          transpose(x, valid);
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const bool up = x[j] > run[c].k;
