@@ -116,14 +116,14 @@ COSPEC_API int cospec_num_sms(void);
  *             with a split planned for a shorter one; it sets no error bit.
  *    No workspace: the KV range of a (sequence, KV head) is split over the
  *    CTAs of one thread-block cluster, whose partial results merge in
- *    distributed shared memory.  Two kernels implement the call: one on
- *    mma.sync tensor-core tiles, and one on tcgen05 (TMEM accumulators, the
- *    query rows as the MMA M dimension, up to 128 rows of a KV head per
- *    CTA, or 256 sharing each K/V tile), used when a KV head has more than 32 query rows (and at most 64
- *    query heads share the KV head).  Batches of up to 64 sequences are
- *    processed longest context first; larger ones in index order (tcgen05:
- *    in reverse when the last context is longer than the first; a caller can
- *    order them).
+ *    distributed shared memory.  Four kernels implement the call: one on
+ *    mma.sync tensor-core tiles, and three on tcgen05 (TMEM accumulators, the
+ *    query rows as the MMA M dimension) for KV heads with more than 32 query rows
+ *    (and at most 64 query heads): 128 rows of a KV head per CTA, 256 per CTA
+ *    sharing each K/V tile, or 256 per pair of CTAs.  The order in which the
+ *    sequences are processed is unspecified and bears on speed alone: longest
+ *    context first up to 64 sequences (384 on CTA pairs), above that index
+ *    order (tcgen05: in reverse when the last context is longer than the first).
  *    Supported: head_dim in {64, 128}; page_size == 16; rows <= 64;
  *    num_q_heads % num_kv_heads == 0; (num_q_heads / num_kv_heads) * rows <= 512.
  * ------------------------------------------------------------------------ */
@@ -166,6 +166,11 @@ typedef struct {
  * for the dimensions. */
 COSPEC_API int cospec_verify_attn_plan(const cospec_attn_dims* dims, int max_ctx, int* kernel,
                                        int* splits);
+
+/* Which of the kernels that plan names: *variant = 0 the mma.sync kernel, 1 tcgen05
+ * with one row tile (128 query rows) per CTA, 2 with two, 3 with two on a pair of
+ * CTAs.  Errors as for cospec_verify_attn_plan. */
+COSPEC_API int cospec_verify_attn_variant(const cospec_attn_dims* dims, int max_ctx, int* variant);
 
 /* Residency model for cospec_verify_attn_plan_model: how many clusters of
  * `splits` CTAs of one attention kernel variant a device keeps resident at

@@ -25,7 +25,8 @@ EXPORTED = ("cospec_status_string", "cospec_last_cuda_error", "cospec_get_device
             "cospec_arbitrate", "cospec_accept_commit", "cospec_lmhead_argmax_features_noalloc",
             "cospec_lmhead_sample_features", "cospec_verify_attn_plan", "cospec_rl_workspace",
             "cospec_rl_advantages", "cospec_verify_attn_plan_model",
-            "cospec_lmhead_logits_features", "cospec_sps_workspace", "cospec_sps_accept", "cospec_accept_commit_launches")
+            "cospec_lmhead_logits_features", "cospec_sps_workspace", "cospec_sps_accept", "cospec_accept_commit_launches",
+            "cospec_verify_attn_variant")
 
 
 class AttnDims(ctypes.Structure):
@@ -77,6 +78,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         "cospec_num_sms": (_i, []),
         "cospec_verify_attn": (_i, [_PDIMS, _i, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp]),
         "cospec_verify_attn_plan": (_i, [_PDIMS, _i, ctypes.POINTER(_i), ctypes.POINTER(_i)]),
+        "cospec_verify_attn_variant": (_i, [_PDIMS, _i, ctypes.POINTER(_i)]),
         "cospec_verify_attn_plan_model": (_i, [_PDIMS, _i, _i, RESIDENT_FN, _vp,
                                                ctypes.POINTER(_i), ctypes.POINTER(_i)]),
         "cospec_rl_workspace": (_sz, [_i, _i]),
@@ -228,6 +230,17 @@ def verify_attn_plan(q, k_pages, page_table, max_ctx: int, kv_stable: bool = Fal
     _check(load_library().cospec_verify_attn_plan(ctypes.byref(dims), int(max_ctx),
                                                   ctypes.byref(kernel), ctypes.byref(splits)))
     return kernel.value, splits.value
+
+
+ATTN_ONE_TILE, ATTN_TWO_TILES, ATTN_CTA_PAIR = 1, 2, 3    # tcgen05 variants (0: mma.sync)
+
+
+def verify_attn_variant(q, k_pages, page_table, max_ctx: int, kv_stable: bool = False) -> int:
+    """Which of the attention kernels cospec_verify_attn would use for these tensors."""
+    dims = attn_dims(q, k_pages, page_table, flags=ATTN_KV_STABLE if kv_stable else 0)
+    variant = ctypes.c_int()
+    _check(load_library().cospec_verify_attn_variant(ctypes.byref(dims), int(max_ctx), ctypes.byref(variant)))
+    return variant.value
 
 
 def verify_attn_plan_model(dims: AttnDims, max_ctx: int, num_sms: int, resident):

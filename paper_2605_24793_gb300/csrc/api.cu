@@ -194,7 +194,8 @@ static int check_attn_dims(const cospec_attn_dims* d) {
 
 // Clusters of S CTAs of a plan's attention variant resident at once (the
 // occupancy query, cached per device; it depends on the variant and its shared
-// memory, not on the grid).
+// memory, not on the grid).  The tcgen05 kernels answer alike: each takes all of
+// an SM's TMEM and at least 118 KB, so one CTA per SM, and clusters of one size fit alike.
 static long long resident_clusters(int D, const AttnPlan& pl, int S, int Hkv, int B, int R) {
   // [dev][D==128][variant][block keys / 16 - 1][S - 1]: count + 1 (0: not yet queried)
   static std::atomic<int> cache[MAX_DEV][2][5][4][16];
@@ -234,6 +235,18 @@ COSPEC_API int cospec_verify_attn_plan(const cospec_attn_dims* d, int max_ctx, i
   const AttnPlan pl = attn_plan(d, max_ctx, sms);
   *kernel = pl.kind;
   *splits = pl.cluster;
+  return COSPEC_OK;
+}
+
+COSPEC_API int cospec_verify_attn_variant(const cospec_attn_dims* d, int max_ctx, int* variant) {
+  const int st = check_attn_dims(d);
+  if (st != COSPEC_OK) return st;
+  CS_CHECK_ARG(variant);
+  CS_CHECK_ARG(max_ctx >= 0 && max_ctx <= d->max_pages_per_seq * d->page_size);
+  const int sms = device_num_sms();
+  if (sms <= 0) return cuda_lookup_failed();
+  const AttnPlan pl = attn_plan(d, max_ctx, sms);
+  *variant = pl.kind == 1 ? 1 + pl.two : 0;
   return COSPEC_OK;
 }
 

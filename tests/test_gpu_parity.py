@@ -157,6 +157,12 @@ ATTN_TC_SPLIT_CASES = [
     (6, 8, 64, 8, 128, [9000, 3000] + _ctx(4, 9), True, 4),       # 48 units
     (1, 8, 64, 8, 128, [6000], False, 12),                        # one wave of 12-CTA clusters
     (20, 8, 64, 8, 128, [33000, 9000] + _ctx(18, 10), False, 2),  # a context past 256 tiles
+    # the halves' maxima swapped (D = 128, up to three tiles per CTA) or not, clusters of eight and more or not
+    (2, 9, 16, 2, 128, [500, 300], True, 2),                      # two tiles per CTA
+    (1, 17, 8, 2, 128, [1537], True, 6),                          # 13 tiles over six
+    (2, 17, 8, 2, 64, [2048, 0], True, 8),                        # head_dim 64, two tiles per CTA
+    (1, 33, 4, 2, 64, [4000], True, 16),                          # the same, clusters of 16
+    (1, 9, 16, 2, 128, [8000], False, 16),                        # four tiles per CTA
 ]
 
 
@@ -180,16 +186,17 @@ EDGE_CTX = [0, 1, 15, 16, 63, 64, 65, 100, 127, 128, 129, 191, 192, 193, 255, 30
 
 
 @pytest.mark.parametrize("full", [False, True], ids=["causal", "full"])
-@pytest.mark.parametrize("R,Hq,Hkv,D", [
-    (33, 32, 8, 128),     # 132 rows: the second row tile has four
-    (53, 32, 8, 128),     # 212 rows
-    (64, 32, 8, 64),      # 256 rows, head_dim 64
-    (64, 24, 8, 128),     # G = 3: row tiles of 42 block rows (126 query rows)
-    (40, 64, 8, 128),     # G = 8: a group of two row tiles and one of a single tile
-    (20, 32, 8, 128),     # 80 rows: the one-tile kernel, unsplit
-    (32, 16, 8, 64),      # 64 rows, head_dim 64
+@pytest.mark.parametrize("R,Hq,Hkv,D,variant", [
+    (33, 32, 8, 128, C.ATTN_TWO_TILES),     # 132 rows: the second row tile has four
+    (53, 32, 8, 128, C.ATTN_TWO_TILES),     # 212 rows
+    (64, 32, 8, 64, C.ATTN_TWO_TILES),      # 256 rows, head_dim 64
+    (64, 24, 8, 128, C.ATTN_TWO_TILES),     # G = 3: row tiles of 42 block rows (126 query rows)
+    (40, 64, 8, 128, C.ATTN_TWO_TILES),     # G = 8: a group of two row tiles and one of a single tile
+    (40, 64, 8, 64, C.ATTN_TWO_TILES),      # the same, head_dim 64
+    (20, 32, 8, 128, C.ATTN_ONE_TILE),      # 80 rows, unsplit
+    (32, 16, 8, 64, C.ATTN_ONE_TILE),       # 64 rows, head_dim 64
 ])
-def test_verify_attention_tile_edges(R, Hq, Hkv, D, full):
+def test_verify_attention_tile_edges(R, Hq, Hkv, D, variant, full):
     """One and two row tiles per CTA at every key remainder (more than 128 rows on 128 or more
     (sequence, head) units of a few tiles take two).  bf16 outputs of probabilities rounded to bf16:
     the usual tolerance."""
@@ -197,6 +204,7 @@ def test_verify_attention_tile_edges(R, Hq, Hkv, D, full):
     rng = np.random.default_rng(R * 100 + Hq + D)
     t = _paged_case(rng, B, R, Hq, Hkv, D, EDGE_CTX, True)
     assert C.verify_attn_plan(t["q"], t["k_pages"], t["page_table"], max(EDGE_CTX)) == (C.ATTN_TCGEN05, 1)
+    assert C.verify_attn_variant(t["q"], t["k_pages"], t["page_table"], max(EDGE_CTX)) == variant
     out = torch.empty_like(t["q"])
     C.verify_attn(t["q"], t["k_blk"], t["v_blk"], t["k_pages"], t["v_pages"], t["page_table"],
                   t["ctx_len"], out, max(EDGE_CTX), block_full=full)
@@ -1026,7 +1034,7 @@ PAIR_CTX = [0, 1, 15, 16, 17, 63, 64, 65, 127, 128, 129, 191, 192, 255, 256, 257
 
 @pytest.mark.parametrize("full", [False, True], ids=["causal", "full"])
 @pytest.mark.parametrize("B,R,Hq,Hkv", [
-    (100, 33, 8, 2), (100, 53, 8, 2), (100, 64, 8, 2), (100, 17, 16, 2), (100, 64, 16, 2), (420, 33, 4, 1),
+    (100, 33, 8, 2), (100, 53, 8, 2), (100, 64, 8, 2), (100, 17, 16, 2), (120, 64, 16, 2), (420, 33, 8, 2),
     (420, 33, 32, 8),
 ])
 def test_verify_attention_pair_edges(B, R, Hq, Hkv, full):
@@ -1035,6 +1043,7 @@ def test_verify_attention_pair_edges(B, R, Hq, Hkv, full):
     ctx = [PAIR_CTX[(i * 7) % len(PAIR_CTX)] for i in range(B)]
     t = _paged_case(rng, B, R, Hq, Hkv, D, ctx, True)
     assert C.verify_attn_plan(t["q"], t["k_pages"], t["page_table"], max(ctx)) == (C.ATTN_TCGEN05, 1)
+    assert C.verify_attn_variant(t["q"], t["k_pages"], t["page_table"], max(ctx)) == C.ATTN_CTA_PAIR
     out = torch.empty_like(t["q"])
     for b in range(B):                   # the rest of each last page is NaN
         if ctx[b] % 16:
@@ -1066,6 +1075,7 @@ def test_verify_attention_pair_skips_only_the_bad_sequence():
     rng = np.random.default_rng(53)
     ctx = [640 - 3 * i for i in range(B)]
     t = _paged_case(rng, B, R, Hq, Hkv, D, ctx, True)
+    assert C.verify_attn_variant(t["q"], t["k_pages"], t["page_table"], 640) == C.ATTN_CTA_PAIR
     call = lambda c, o: C.verify_attn(t["q"], t["k_blk"], t["v_blk"], t["k_pages"], t["v_pages"],
                                       t["page_table"], c, o, 640)
     good, out = torch.empty_like(t["q"]), torch.full_like(t["q"], float("nan"))
