@@ -146,17 +146,8 @@ CS_DEV uint64_t l2_policy_evict_last() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-// 2-D tiled load: box at element coordinates (x = innermost, y) into shared
+// 3-D and 4-D tiled loads: box at element coordinates (x = innermost, y, ...) into shared
 // memory, completion signalled on `bar` (transaction bytes).
-CS_DEV void tma_load_2d(uint32_t dst, const void* map, uint64_t* bar, int x, int y,
-                        uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(dst),
-      "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy)
-      : "memory");
-}
-
 CS_DEV void tma_load_3d(uint32_t dst, const void* map, uint64_t* bar, int x, int y, int z,
                         uint64_t policy) {
   asm volatile(
@@ -270,22 +261,6 @@ CS_DEV void tmem_alloc_pair(uint32_t* dst_smem, uint32_t ncols) {   // one warp 
 CS_DEV void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
                : "memory");
-}
-CS_DEV void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                           uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// Arrive on the barrier at this offset in both CTAs once every pair MMA issued so far is done.
-CS_DEV void umma_commit_pair(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "h"((uint16_t)3)
-      : "memory");
 }
 // 2-D tiled load into this CTA's shared memory whose bytes are counted on a barrier of either CTA of
 // the pair (`bar_cluster`: a cluster address).
