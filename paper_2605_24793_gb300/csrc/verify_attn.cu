@@ -678,18 +678,19 @@ int variant_mt(int NR) {   // NR <= 64
 // rows per KV head, groups of 128 (one MMA row tile per CTA, 1 to 16 splits) or of 256, unsplit (two
 // row tiles sharing a K/V stream in one CTA, or a persistent CTA pair for head dimension 128), by the
 // smallest estimated time.  The estimates are as measured on GB300 (us): a CTA 7 + 0.94 per 128-key
-// tile, 4 more when split (3 where the units are a quarter of a wave); two row tiles 7.5 + 1.9 per tile, whole waves of either at 15 % more from
-// the second on; a pair 3 and 4.4 + 0.79 per tile for each of its units.  They are put together for
+// tile, 4 more when split (3 where the units are a quarter of a wave); two row tiles 7.5 + 1.9 per
+// tile, whole waves of either at 15 % more from the second on; a pair 3 and 4.4 + 0.79 per tile for
+// each of its units.  They are put together for
 // equal contexts (whole waves, whole rounds of units) and for contexts that average 0.65 of the
 // longest (the longest CTA or unit, or the work spread over the resident clusters), weighted 0.35 to
 // 0.65 since only the longest context is known here.  Against the rule before (128 rows per group,
 // powers of two near one wave of CTAs), us per launch: K = 25 regions (212 rows) at batch 4, 4096 keys
 // 37.8 -> 26.6, batch 8 57.5 -> 32.0, batch 16 83.7 -> 60.9, batch 16 at 2048..4096 keys 66.3 -> 48.5, at
 // 512 keys 23.9 -> 15.9; 208 rows, batch 32 at 2048..8192 keys 184.8 -> 133; K = 7 regions (68 rows) at
-// batch 16, 4096 keys 56 -> 44.  Over 4113 sizes (both head dimensions, 36 to 512 rows, batches 1 to 100, 64 to
-// 8192 keys) 0.53 to 1.08 of the time, 0.88 on average, the slowest by 0.5 us at 100 keys.  The same figures
-// serve head dimension 64, whose tiles take as long here (2 KB boxes): one-tile launches above a quarter of a
-// wave come within 0.7 % of the best split tried, 0.5 % at 128.
+// batch 16, 4096 keys 56 -> 44.  Over 5555 launches (both head dimensions, 36 to 512 rows, batches 1 to 100,
+// 64 to 8192 keys) 0.88 of the time on average; of those slower by 5 % the ones timed again with their buffers
+// in the same place were so by at most 0.5 us.  The same figures serve head dimension 64, whose tiles take as long here (2 KB boxes): one-tile launches
+// above a quarter of a wave come within 0.7 % of the best split tried on average, 0.5 % at 128.
 static AttnPlan plan_tcq(const AttnPlan& base, int B, int R, int Hkv, int D, int max_ctx,
                          const ResidentFn& resident) {
   const int tiles = (max_ctx + 127) / 128;
