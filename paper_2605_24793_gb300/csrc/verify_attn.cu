@@ -678,7 +678,7 @@ int variant_mt(int NR) {   // NR <= 64
 // rows per KV head, groups of 128 (one MMA row tile per CTA, 1 to 16 splits) or of 256, unsplit (two
 // row tiles sharing a K/V stream in one CTA, or a persistent CTA pair for head dimension 128), by the
 // smallest estimated time.  The estimates are as measured on GB300 (us): a CTA 7 + 0.94 per 128-key
-// tile, 4 more when split (3 where the units are a quarter of a wave); two row tiles 7.5 + 1.9 per
+// tile, 3.25 more when split (3 where the units are a quarter of a wave); two row tiles 7.5 + 1.9 per
 // tile, whole waves of either at 15 % more from the second on; a pair 3 and 4.4 + 0.79 per tile for
 // each of its units.  They are put together for
 // equal contexts (whole waves, whole rounds of units) and for contexts that average 0.65 of the
@@ -718,7 +718,7 @@ static AttnPlan plan_tcq(const AttnPlan& base, int B, int R, int Hkv, int D, int
         longest = 3.0 + (4.4 + 0.79 * tiles);
         spread = 3.0 + (double)pl.units / fit * (4.4 + 0.79 * 0.65 * tiles);
       } else {
-        const double per_tile = two ? 1.9 : 0.94, start = two ? 7.5 : s == 1 ? 7.0 : pl.units * 4 <= one ? 10.0 : 11.0;
+        const double per_tile = two ? 1.9 : 0.94, start = two ? 7.5 : s == 1 ? 7.0 : pl.units * 4 <= one ? 10.0 : 10.25;
         // (split, the block counts as 0.6 of a tile on the last CTA: 16 tiles take five CTAs, not four)
         const int most = (tiles + s - 1) / s, rest = tiles - (s - 1) * most > 0 ? tiles - (s - 1) * most : 0;
         longest = start + per_tile * (s > 1 && rest + 0.6 > most ? rest + 0.6 : most);

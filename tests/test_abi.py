@@ -123,6 +123,7 @@ PLAN_CASES = [
     ((64, 8, 32, 8, 128, 32768, 1), (C.ATTN_MMA_SYNC, 2)),  # Llama-3-8B, batch 64
     ((8, 26, 32, 8, 128, 1024, 1), (C.ATTN_TCGEN05, 1)),    # 64 units of 8 tiles: unsplit 15.3 us, 2 splits 16.8
     ((32, 64, 4, 2, 128, 1024, 1), (C.ATTN_TCGEN05, 1)),    # the same with 128 rows: 15.9 against 17.8
+    ((16, 26, 32, 8, 128, 7876, 1), (C.ATTN_TCGEN05, 2)),   # K = 25 at 2048..7876 keys: 65.3 us, unsplit 68.0
     ((1, 64, 32, 8, 64, 700, 1), (C.ATTN_TCGEN05, 3)),      # 16 units of 6 tiles: 10.1 us, unsplit 10.9
     ((1, 33, 64, 8, 128, 2048, 1), (C.ATTN_TCGEN05, 5)),    # 16 tiles over five CTAs: the last has the block alone
 ]
